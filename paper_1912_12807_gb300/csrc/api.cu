@@ -228,6 +228,7 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
                                  cudaMemcpyHostToDevice, s));
     }
     PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
+    if (fil->nbits == 1 && plan->nsub == 0 && ck <= 255) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
     // the boxcar table of the downsampled rows (exact plans only)
     if (plan->nsub == 0) {
         size_t need_bx = 0;
@@ -267,9 +268,10 @@ pss_status upload_input(pss_ctx* ctx, const pss_fil_desc* fil, const void* data,
     return PSS_OK;
 }
 
-// Unpack/transpose the file into ctx->xcm (kernel launch only).
+// Unpack/transpose the file into ctx->xcm, or, as rows of bits, into
+// ctx->xbits (kernel launches only).
 pss_status enqueue_prep(pss_ctx* ctx, const pss_fil_desc* fil, const uint8_t* src, int32_t ck, int64_t pitch,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool bytes = true, bool bits = false) {
     PrepArgs pa;
     pa.src = src;
     pa.nchan = fil->nchan;
@@ -281,8 +283,11 @@ pss_status enqueue_prep(pss_ctx* ctx, const pss_fil_desc* fil, const uint8_t* sr
     pa.xcm = (uint8_t*)ctx->xcm.p;
     pa.pitch = pitch;
     ProfScope ps(ctx, 0, s);
-    PSS_CUDA(launch_prep(pa, s));
-    ctx->bx_ds = 0;  // the boxcar table no longer matches the channel-major data
+    if (bits) PSS_CUDA(launch_prep_bits(pa, (uint8_t*)ctx->xbits.p, b1_pitch(fil->nsamp), s));
+    if (bytes) {
+        PSS_CUDA(launch_prep(pa, s));
+        ctx->bx_ds = 0;  // the boxcar table no longer matches the channel-major data
+    }
     return PSS_OK;
 }
 
@@ -298,8 +303,7 @@ pss_status stage_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
 
 // max over the dedispersion kernel's groups of consecutive trials and over
 // channels of (dmax - dmin)
-int32_t delay_spread(const int32_t* d, int64_t nb, int32_t ck) {
-    const int G = dedisp_group_trials();
+int32_t delay_spread(const int32_t* d, int64_t nb, int32_t ck, int G = dedisp_group_trials()) {
     int32_t sp = 0;
     for (int64_t g = 0; g < nb; g += G) {
         const int64_t ge = std::min<int64_t>(nb, g + G);
@@ -365,15 +369,92 @@ SubBatch sub_batch(const pss_plan* plan, const SubTab& T, int32_t ck, int64_t dm
     return B;
 }
 
+// How one DM batch of an exact plan is dedispersed.
+enum DdKind {
+    DD_DIRECT,  // k_dedisp, or the boxcar table (enqueue_dedisp's rule)
+    DD_SHARED,  // shared sums (k_dedisp_sh), tables in ctx->ddtab[which]
+    DD_BITS,    // bit-sliced 1-bit samples (k_dedisp_b1)
+};
+struct DdBatch {
+    int kind = DD_DIRECT;
+    int which = 0;
+    size_t off = 0, chunk_off = 0, chan_off = 0;
+    int32_t spread = 0, group = 0;  // bit-sliced: trials per CTA and their delay spread
+};
+
+// Choose a batch's kernel (delays [nb][ck]); shared-sum tables are appended to `host`.
+void dd_choose(const Tune& tune, const pss_fil_desc* fil, const StageInfo& st, const int32_t* delays, int32_t nb,
+               int32_t ck, int which, std::vector<uint8_t>* host, DdBatch* d) {
+    d->kind = DD_DIRECT;
+    d->which = which;
+    if (fil->nbits == 1) {
+        // 32 trials share a staged tile, 16 where that leaves fewer than two CTAs for each of about 150 SMs
+        const int64_t tiles = (st.nv * st.ds + 4095) / 4096;
+        d->group = tiles * ((nb + 31) / 32) >= 300 ? 32 : 16;
+        d->spread = delay_spread(delays, nb, ck, d->group);
+        int KW, rowb;
+        size_t shm;
+        if (b1_sizes(d->spread, ck, d->group, &KW, &rowb, &shm)) d->kind = DD_BITS;
+        return;
+    }
+    if (bx_use(tune, st.ds) && ck <= 65535) return;
+    if (st.ds > 64 || nb < 8) return;
+    DdTables t;
+    if (!dd_tables(delays, nb, ck, &t)) return;
+    // Shared sums where they take at most 1.2 shared-memory wavefronts per channel, trial and 128 samples (the
+    // direct kernel: 1, and five instructions).  Measured: 0.95 (256 channels, 0.5 pc cm^-3 steps) 2.45 against
+    // 3.91 ms, 1.14 (1 pc cm^-3 steps) 1.23 against 1.57 ms, 1.31 (64 channels, where most of 32 trials have
+    // patterns of their own) 54.7 against 51.2 us.
+    if (t.cost > 1.2 * (double)nb * ck) return;
+    d->kind = DD_SHARED;
+    d->off = (host->size() + 255) & ~size_t(255);
+    d->chunk_off = t.chunk_off;
+    d->chan_off = t.chan_off;
+    host->resize(d->off + t.bytes.size());
+    memcpy(host->data() + d->off, t.bytes.data(), t.bytes.size());
+}
+
+// Put the batches' tables on the device (waits: `host` is the caller's).  The
+// set-up kept for that buffer goes first: its tables are overwritten.
+pss_status dd_upload(pss_ctx* ctx, int which, const std::vector<uint8_t>& host, cudaStream_t s) {
+    if (host.empty()) return PSS_OK;
+    (which == 0 ? ctx->path_cache : ctx->dd_cache).reset();
+    PSS_TRY(ctx->ddtab[which].ensure(host.size()));
+    PSS_CUDA(cudaMemcpyAsync(ctx->ddtab[which].p, host.data(), host.size(), cudaMemcpyHostToDevice, s));
+    PSS_CUDA(cudaStreamSynchronize(s));
+    return PSS_OK;
+}
+
 // Dedisperse trials [b0, b0 + nb) of one stage into rows of out_stride
 // (float out_f with per-trial sums, or int32 out_i): the exact kernel, or,
 // for a two-stage plan, stage 1 into `subu` and stage 2 from it.  `spread`
 // is the exact kernel's delay spread; `SB` the two-stage launch sizes.
 pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_t pitch, const SubTab& T,
                           const StageInfo& st, int64_t dm_begin, int64_t b0, int32_t nb, int32_t spread,
-                          const SubBatch& SB, void* subu, float* out_f, int32_t* out_i, int64_t out_stride,
-                          unsigned long long* sums, cudaStream_t s) {
+                          const SubBatch& SB, const DdBatch& dd, void* subu, float* out_f,
+                          int32_t* out_i, int64_t out_stride, unsigned long long* sums, cudaStream_t s) {
     const int32_t* base = (const int32_t*)ctx->delays_dev.p;
+    if (!T.on && dd.kind == DD_BITS) {
+        B1Args ba{};
+        ba.xb = (const uint8_t*)ctx->xbits.p;
+        ba.pitchb = b1_pitch(plan->nsamp);
+        ba.ck = ck;
+        ba.G = dd.group;
+        ba.delays = base + ck + (b0 - dm_begin) * ck;
+        ba.nb = nb;
+        ba.nv = st.nv;
+        ba.lds = ilog2(st.ds);
+        ba.out_f = out_f;
+        ba.out_i = out_i;
+        ba.out_stride = out_stride;
+        ba.vec4 = out_f && out_stride % 4 == 0 && ((uintptr_t)out_f & 15) == 0;
+        ba.sums = sums;
+        ba.err = (int*)ctx->errflag.p;
+        ba.wait_polls = ctx->wait_polls;
+        ProfScope ps(ctx, 1, s);
+        PSS_CUDA(launch_dedisp_b1(ba, dd.spread, s));
+        return PSS_OK;
+    }
     // downsampled row: one boxcar table per ds (built once per file and ds), then one term per channel;
     // a few trials alone do not pay for building the table
     if (!T.on && bx_use(ctx->tune, st.ds) && ck <= 65535 && ctx->bx.bytes >= bx_table_bytes(ck, plan->nsamp, st.ds) &&
@@ -407,6 +488,28 @@ pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_
         ba.out_stride = out_stride;
         ba.sums = sums;
         PSS_CUDA(launch_dedisp_bx(ba, s));
+        return PSS_OK;
+    }
+    if (!T.on && dd.kind == DD_SHARED) {
+        DdArgs da{};
+        da.xcm = (const uint8_t*)ctx->xcm.p;
+        da.pitch = pitch;
+        da.ck = ck;
+        da.tab = (const uint8_t*)ctx->ddtab[dd.which].p + dd.off;
+        da.chunk_off = dd.chunk_off;
+        da.chan_off = dd.chan_off;
+        da.nb = nb;
+        da.nv = st.nv;
+        da.lds = ilog2(st.ds);
+        da.out_f = out_f;
+        da.out_i = out_i;
+        da.out_stride = out_stride;
+        da.vec4 = out_f && out_stride % 4 == 0 && ((uintptr_t)out_f & 15) == 0;
+        da.sums = sums;
+        da.err = (int*)ctx->errflag.p;
+        da.wait_polls = ctx->wait_polls;
+        ProfScope ps(ctx, 1, s);
+        PSS_CUDA(launch_dedisp_sh(da, s));
         return PSS_OK;
     }
     if (!T.on) {
@@ -677,6 +780,7 @@ struct BatchDesc {
     int32_t spread;    // delay spread the dedispersion launch is sized for
     int64_t out_off;   // packed output offset (spectrum / plane modes)
     SubBatch sub;      // two-stage launch sizes
+    DdBatch dd;        // shared-sum tables
 };
 
 // Everything the kernel sequence needs, computed on the host once.
@@ -688,6 +792,7 @@ struct PathSetup {
     std::vector<BatchDesc> batches;
     std::vector<HarmArgs> harm;  // per stage: thresholds and f_lo cuts
     int64_t dev_cap = 0;
+    bool need_bytes = false, need_bits = false;  // unpacked forms of the file its batches read
 };
 
 // Trials per batch for a stage of nfft-point spectra: as many as fit in
@@ -762,6 +867,84 @@ std::string path_key(const pss_plan* plan, const pss_fil_desc* fil, const pss_se
     return k;
 }
 
+// Host set-up of a plain dedispersion (pss_dedisperse, pss_single_pulse) of
+// [dm_begin, dm_end): input tables, DM batches, shared-sum tables and the
+// stage-1 buffer, kept like PathCache while the request is the same and the
+// device tables are still the ones uploaded for it.
+enum DdUse { DD_DEDISPERSE, DD_SINGLE_PULSE };
+
+struct DdSetup {
+    std::string key;
+    uint64_t gen = 0;
+    int32_t ck = 0;
+    int64_t pitch = 0;
+    SubTab T;
+    std::vector<BatchDesc> batches;  // out_off: samples of the trials before, packed
+    size_t need_subu = 0;
+    bool need_bytes = false, need_bits = false;
+};
+
+pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin, int64_t dm_end,
+                        DdUse use, cudaStream_t s, std::shared_ptr<DdSetup>* out) {
+    const pss_search_cfg none{};
+    std::string key = path_key(plan, fil, &none, dm_begin, dm_end, MODE_SPECTRUM, (int64_t)use, 0, ctx->tune);
+    key_put(&key, ctx->tune.bx_min);
+    auto kept = std::static_pointer_cast<DdSetup>(ctx->dd_cache);
+    if (kept && kept->key == key && dm_end > dm_begin) {
+        if (kept->gen != ctx->delays_gen) {  // another request's delays are on the device
+            SubTab T;
+            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &kept->ck, &kept->pitch, &T));
+            kept->gen = ctx->delays_gen;
+        }
+        if (kept->need_subu) PSS_TRY(ctx->subu.ensure(kept->need_subu));
+        *out = kept;
+        return PSS_OK;
+    }
+    auto D = std::make_shared<DdSetup>();
+    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T));
+    D->need_bytes = D->T.on;
+    const std::vector<int32_t> hd = D->T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
+    std::vector<uint8_t> dd_host;
+    int64_t off = 0;
+    for (size_t si = 0; si < plan->stages.size(); ++si) {
+        const StageInfo& st = plan->stages[si];
+        const int64_t lo = std::max<int64_t>(dm_begin, st.first);
+        const int64_t hi = std::min<int64_t>(dm_end, st.first + st.n_dm);
+        if (lo >= hi) continue;
+        // single pulses: up to 1 GiB of int32 series; two-stage plans: whole groups
+        int64_t B = use == DD_SINGLE_PULSE ? std::max<int64_t>(1, std::min<int64_t>(1024, ((int64_t)1 << 28) / st.nv)) : 1024;
+        if (D->T.on) {
+            if (use == DD_DEDISPERSE) B = std::max<int64_t>(1, std::min<int64_t>(B, 256 / plan->sub_group) * plan->sub_group);
+            else if (B > plan->sub_group) B = B / plan->sub_group * plan->sub_group;
+        }
+        for (int64_t b0 = lo; b0 < hi; b0 += B) {
+            BatchDesc d{};
+            d.stage = (int32_t)si;
+            d.b0 = b0;
+            d.nb = (int32_t)std::min<int64_t>(B, hi - b0);
+            if (D->T.on) {
+                d.sub = sub_batch(plan, D->T, D->ck, dm_begin, b0, d.nb, st.nv, st.ds);
+                D->need_subu = std::max(D->need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
+            } else {
+                const int32_t* rows = hd.data() + (size_t)(b0 - dm_begin) * D->ck;
+                d.spread = delay_spread(rows, d.nb, D->ck);
+                dd_choose(ctx->tune, fil, st, rows, d.nb, D->ck, 1, &dd_host, &d.dd);
+                (d.dd.kind == DD_BITS ? D->need_bits : D->need_bytes) = true;
+            }
+            d.out_off = off;
+            off += (int64_t)d.nb * st.nv;
+            D->batches.push_back(d);
+        }
+    }
+    if (D->need_subu) PSS_TRY(ctx->subu.ensure(D->need_subu));
+    PSS_TRY(dd_upload(ctx, 1, dd_host, s));
+    D->key.swap(key);
+    D->gen = ctx->delays_gen;
+    ctx->dd_cache = D;
+    *out = D;
+    return PSS_OK;
+}
+
 pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, const pss_search_cfg* cfg,
                       int64_t dm_begin, int64_t dm_end, Mode mode, cudaStream_t s, int64_t dev_cap, PathSetup* P,
                       int64_t max_b = 0) {
@@ -778,6 +961,8 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
         P->harm.clear();
     }
     P->dev_cap = dev_cap;
+    // (MODE_GAINS: the refinement also reads the byte rows, channel by channel)
+    if (!hit) P->need_bytes = P->sub.on || mode == MODE_GAINS || dm_end == dm_begin;
     if (dm_end == dm_begin) return PSS_OK;
     PSS_TRY(ensure_templates(ctx, cfg, s));
     P->nz = nz_of(cfg);
@@ -801,6 +986,7 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
         if (st.n_dm > 0) PSS_TRY(ensure_passtw(ctx, st.nfft / 2, ctx->tune.split_for(st.nfft / 2), s));
     size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, need_subu = 0;
     int64_t out_off = 0;
+    std::vector<uint8_t> dd_host;
     if (hit) {
         need_series = pc->need[0];
         need_fft = pc->need[1];
@@ -840,13 +1026,17 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
                 d.sub = sub_batch(plan, P->sub, P->ck, dm_begin, b0, d.nb, st.nv, st.ds);
                 need_subu = std::max(need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
             } else {
-                d.spread = delay_spread(hd.data() + (size_t)(b0 - dm_begin) * P->ck, d.nb, P->ck);
+                const int32_t* rows = hd.data() + (size_t)(b0 - dm_begin) * P->ck;
+                d.spread = delay_spread(rows, d.nb, P->ck);
+                dd_choose(ctx->tune, fil, st, rows, d.nb, P->ck, 0, &dd_host, &d.dd);
+                (d.dd.kind == DD_BITS ? P->need_bits : P->need_bytes) = true;
             }
             d.out_off = out_off;
             out_off += (mode == MODE_SPECTRUM) ? (int64_t)d.nb * M : (mode == MODE_PLANE) ? (int64_t)d.nb * P->nz * nfft : 0;
             P->batches.push_back(d);
         }
     }
+    if (!hit) PSS_TRY(dd_upload(ctx, 0, dd_host, s));
     PSS_TRY(ctx->series.ensure(need_series));
     if (need_subu) PSS_TRY(ctx->subu.ensure(need_subu));
     PSS_TRY(ctx->sums.ensure(need_sums));
@@ -874,14 +1064,14 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
 pss_status enqueue_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, const uint8_t* src,
                         const pss_search_cfg* cfg, int64_t dm_begin, const PathSetup& P, Mode mode, Outputs outs,
                         cudaStream_t s, bool snapshots = false) {
-    PSS_TRY(enqueue_prep(ctx, fil, src, P.ck, P.pitch, s));
+    PSS_TRY(enqueue_prep(ctx, fil, src, P.ck, P.pitch, s, P.need_bytes, P.need_bits));
     if (P.batches.empty()) return PSS_OK;
     if (mode == MODE_SEARCH) PSS_CUDA(cudaMemsetAsync(ctx->counter.p, 0, sizeof(unsigned long long), s));
     for (const BatchDesc& d : P.batches) {
         const StageInfo& st = plan->stages[d.stage];
         const int64_t nfft = st.nfft, M = nfft / 2;
         PSS_CUDA(cudaMemsetAsync(ctx->sums.p, 0, (size_t)d.nb * 8, s));
-        PSS_TRY(enqueue_dedisp(ctx, plan, P.ck, P.pitch, P.sub, st, dm_begin, d.b0, d.nb, d.spread, d.sub,
+        PSS_TRY(enqueue_dedisp(ctx, plan, P.ck, P.pitch, P.sub, st, dm_begin, d.b0, d.nb, d.spread, d.sub, d.dd,
                                ctx->subu.p, (float*)ctx->series.p, nullptr, nfft,
                                (unsigned long long*)ctx->sums.p, s));
         const bool fused = (mode == MODE_SEARCH || mode == MODE_PLANE) && cfg->zmax == 0 && nfft == (int64_t(1) << 18) &&
@@ -1736,7 +1926,7 @@ void pss_ctx_destroy(pss_ctx* c) {
     if (!c) return;
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
-    DevBuf* bufs[] = {&c->fil_dev, &c->xcm, &c->delays_dev, &c->subu, &c->sp_series, &c->sp_mom, &c->sp_ev,
+    DevBuf* bufs[] = {&c->fil_dev, &c->xcm, &c->xbits, &c->delays_dev, &c->ddtab[0], &c->ddtab[1], &c->subu, &c->sp_series, &c->sp_mom, &c->sp_ev,
                       &c->fold_buf, &c->bx, &c->mf_fil, &c->mf_xcm, &c->mf_work, &c->series, &c->sums, &c->fftA, &c->fftB,
                       &c->spec, &c->plane, &c->cands, &c->counter, &c->taps, &c->ftaps, &c->tapinfo, &c->errflag,
                       &c->twid, &c->chan_spec, &c->refine_gains, &c->refine_dtau, &c->refine_pts, &c->refine_out};
@@ -1873,33 +2063,15 @@ pss_status pss_dedisperse(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc
     if (!out && dm_end > dm_begin) return fail(PSS_EINVAL, "pss_dedisperse: null out");
     PSS_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t s = pick_stream(ctx, stream);
-    int32_t ck = 0;
-    int64_t pitch = 0;
-    SubTab T;
-    PSS_TRY(stage_input(ctx, plan, fil, data, data_on_device, dm_begin, dm_end, s, &ck, &pitch, &T));
-    const std::vector<int32_t> hd = T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
-    int64_t off = 0;
-    for (size_t si = 0; si < plan->stages.size(); ++si) {
-        const StageInfo& st = plan->stages[si];
-        const int64_t lo = std::max<int64_t>(dm_begin, st.first);
-        const int64_t hi = std::min<int64_t>(dm_end, st.first + st.n_dm);
-        if (lo >= hi) continue;
-        int64_t B = 1024;
-        if (T.on) B = std::max<int64_t>(1, std::min<int64_t>(B, 256 / plan->sub_group) * plan->sub_group);
-        for (int64_t b0 = lo; b0 < hi; b0 += B) {
-            const int32_t nb = (int32_t)std::min<int64_t>(B, hi - b0);
-            int32_t spread = 0;
-            SubBatch SB;
-            if (T.on) {
-                SB = sub_batch(plan, T, ck, dm_begin, b0, nb, st.nv, st.ds);
-                PSS_TRY(ctx->subu.ensure((size_t)plan->nsub * SB.ngb * SB.stride1 * 4 + subsum_slack_bytes(SB.spread2)));
-            } else {
-                spread = delay_spread(hd.data() + (size_t)(b0 - dm_begin) * ck, nb, ck);
-            }
-            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, dm_begin, b0, nb, spread, SB, ctx->subu.p, nullptr,
-                                   out + off, st.nv, nullptr, s));
-            off += (int64_t)nb * st.nv;
-        }
+    std::shared_ptr<DdSetup> D;
+    PSS_TRY(setup_dedisp(ctx, plan, fil, dm_begin, dm_end, DD_DEDISPERSE, s, &D));
+    const uint8_t* src = nullptr;
+    PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
+    PSS_TRY(enqueue_prep(ctx, fil, src, D->ck, D->pitch, s, D->need_bytes, D->need_bits));
+    for (const BatchDesc& d : D->batches) {
+        const StageInfo& st = plan->stages[d.stage];
+        PSS_TRY(enqueue_dedisp(ctx, plan, D->ck, D->pitch, D->T, st, dm_begin, d.b0, d.nb, d.spread, d.sub, d.dd,
+                               ctx->subu.p, nullptr, out + d.out_off, st.nv, nullptr, s));
     }
     return PSS_OK;
 }
@@ -1922,39 +2094,26 @@ pss_status pss_single_pulse(pss_ctx* ctx, const pss_plan* plan, const pss_fil_de
     if (!out && cap > 0) return fail(PSS_EINVAL, "pss_single_pulse: null out");
     PSS_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t s = pick_stream(ctx, stream);
-    int32_t ck = 0;
-    int64_t pitch = 0;
-    SubTab T;
-    PSS_TRY(stage_input(ctx, plan, fil, data, data_on_device, dm_begin, dm_end, s, &ck, &pitch, &T));
-    const std::vector<int32_t> hd = T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
+    std::shared_ptr<DdSetup> D;
+    PSS_TRY(setup_dedisp(ctx, plan, fil, dm_begin, dm_end, DD_SINGLE_PULSE, s, &D));
+    const uint8_t* src = nullptr;
+    PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
+    PSS_TRY(enqueue_prep(ctx, fil, src, D->ck, D->pitch, s, D->need_bytes, D->need_bits));
     PSS_TRY(ctx->counter.ensure(sizeof(unsigned long long)));
     int64_t devcap = std::max<int64_t>((int64_t)ctx->sp_ev.bytes / (int64_t)sizeof(SpRaw), 1 << 16);
     PSS_TRY(ctx->sp_ev.ensure((size_t)devcap * sizeof(SpRaw)));
     std::vector<SpRaw> raw;
     std::vector<unsigned long long> mom_all((size_t)2 * (dm_end - dm_begin));
-    for (size_t si = 0; si < plan->stages.size(); ++si) {
-        const StageInfo& st = plan->stages[si];
-        const int64_t lo = std::max<int64_t>(dm_begin, st.first);
-        const int64_t hi = std::min<int64_t>(dm_end, st.first + st.n_dm);
-        if (lo >= hi) continue;
-        // trials per batch: up to 1 GiB of int32 series, whole groups for two-stage plans
-        int64_t B = std::max<int64_t>(1, std::min<int64_t>(1024, ((int64_t)1 << 28) / st.nv));
-        if (T.on && B > plan->sub_group) B = B / plan->sub_group * plan->sub_group;
-        PSS_TRY(ctx->sp_series.ensure((size_t)std::min<int64_t>(B, hi - lo) * st.nv * sizeof(int32_t)));
-        PSS_TRY(ctx->sp_mom.ensure((size_t)(2 + SP_MAXW) * std::min<int64_t>(B, hi - lo) * sizeof(unsigned long long)));
-        for (int64_t b0 = lo; b0 < hi; b0 += B) {
-            const int32_t nb = (int32_t)std::min<int64_t>(B, hi - b0);
-            int32_t spread = 0;
-            SubBatch SB;
-            if (T.on) {
-                SB = sub_batch(plan, T, ck, dm_begin, b0, nb, st.nv, st.ds);
-                PSS_TRY(ctx->subu.ensure((size_t)plan->nsub * SB.ngb * SB.stride1 * 4 + subsum_slack_bytes(SB.spread2)));
-            } else {
-                spread = delay_spread(hd.data() + (size_t)(b0 - dm_begin) * ck, nb, ck);
-            }
+    for (const BatchDesc& d : D->batches) {
+        const StageInfo& st = plan->stages[d.stage];
+        {
+            const int64_t b0 = d.b0;
+            const int32_t nb = d.nb;
+            PSS_TRY(ctx->sp_series.ensure((size_t)nb * st.nv * sizeof(int32_t)));
+            PSS_TRY(ctx->sp_mom.ensure((size_t)(2 + SP_MAXW) * nb * sizeof(unsigned long long)));
             int32_t* ser = (int32_t*)ctx->sp_series.p;
-            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, dm_begin, b0, nb, spread, SB, ctx->subu.p, nullptr,
-                                   ser, st.nv, nullptr, s));
+            PSS_TRY(enqueue_dedisp(ctx, plan, D->ck, D->pitch, D->T, st, dm_begin, b0, nb, d.spread, d.sub, d.dd,
+                                   ctx->subu.p, nullptr, ser, st.nv, nullptr, s));
             unsigned long long* m1 = (unsigned long long*)ctx->sp_mom.p;
             unsigned long long* m2 = m1 + nb;
             PSS_CUDA(cudaMemsetAsync(m1, 0, (size_t)2 * nb * sizeof(unsigned long long), s));
@@ -1973,7 +2132,7 @@ pss_status pss_single_pulse(pss_ctx* ctx, const pss_plan* plan, const pss_fil_de
             sa.s2 = m2;
             sa.thr_tab = (long long*)(m2 + nb);
             // a sample sums at most 255 (8-bit) or 1 (1-bit) per kept channel and native sample
-            sa.max_value = (long long)ck * (fil->nbits == 8 ? 255 : 1) * st.ds;
+            sa.max_value = (long long)D->ck * (fil->nbits == 8 ? 255 : 1) * st.ds;
             sa.out = (SpRaw*)ctx->sp_ev.p;
             sa.count = (unsigned long long*)ctx->counter.p;
             sa.cap = devcap;
@@ -2092,7 +2251,8 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
                 spread = delay_spread(hd.data() + (size_t)(r.a - lo_dm) * ck, nb, ck);
             }
             int32_t* out = ser + (int64_t)r.row0 * nv_max;
-            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, lo_dm, r.a, nb, spread, SB, ctx->subu.p, nullptr, out,
+            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, lo_dm, r.a, nb, spread, SB, DdBatch(),
+                                   ctx->subu.p, nullptr, out,
                                    nv_max, nullptr, s));
             PSS_CUDA(launch_sp_moments(out, nv_max, st.nv, nb, m1 + r.row0, m2 + r.row0, s));
         }
@@ -2566,7 +2726,7 @@ namespace pss {
 namespace {
 
 size_t ctx_bytes(const pss_ctx* c) {
-    const DevBuf* bufs[] = {&c->fil_dev, &c->xcm, &c->delays_dev, &c->subu, &c->bx, &c->series, &c->sums, &c->fftA,
+    const DevBuf* bufs[] = {&c->fil_dev, &c->xcm, &c->xbits, &c->delays_dev, &c->ddtab[0], &c->ddtab[1], &c->subu, &c->bx, &c->series, &c->sums, &c->fftA,
                             &c->fftB, &c->spec, &c->plane, &c->cands, &c->counter, &c->taps, &c->ftaps, &c->tapinfo,
                             &c->errflag, &c->twid, &c->mf_fil, &c->mf_xcm, &c->mf_work};
     size_t t = 0;
@@ -2833,10 +2993,11 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
         const size_t ng = plan.grp_first.size();
         tables = std::max(tables, (size_t)ck + ng * ck + (size_t)plan.ndm() * plan.nsub + 2 * ng + 2 * plan.nsub + 16);
     }
-    size_t t = buf((size_t)file_bytes(fil)) + buf((size_t)ck * pitch + 64) + buf(tables * sizeof(int32_t)) +
+    size_t t = buf((size_t)file_bytes(fil)) + buf((size_t)ck * pitch + 64) +
+               (fil->nbits == 1 && plan.nsub == 0 && ck <= 255 ? buf(b1_bytes(ck, fil->nsamp)) : 0) + buf(tables * sizeof(int32_t)) +
                buf(sizeof(int)) + buf((size_t)dev_cap * sizeof(pss_raw_cand)) + buf(sizeof(unsigned long long));
     int64_t nfft_max = 0, total_taps = 0;
-    size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, subu = 0, bx = 0;
+    size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, subu = 0, bx = 0, ddt = 0;
     Tune bx_tune;  // the boxcar-table threshold a new context takes (environment included)
     if (const char* f = getenv("PSS_DEDISP_BX_MIN")) bx_tune.bx_min = std::max(0, atoi(f));
     std::vector<int64_t> sizes;
@@ -2849,6 +3010,8 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
             t += buf((size_t)(st.nfft / 2) * sizeof(float2));  // inter-pass twiddles (at most M entries)
         }
         const int64_t B = batch_trials(st.nfft, nz, MODE_SEARCH, st.n_dm);
+        // shared-sum tables of the stage's batches (at most; batches may be smaller than B)
+        if (plan.nsub == 0) ddt += dd_tables_bound(st.n_dm, ck, std::min<int64_t>(B, std::max<int64_t>(1, pipeline_batch(plan.ndm()))));
         if (plan.nsub > 0) {
             // stage-1 rows: groups touched by a batch x subbands x (N_v ds + largest D, padded)
             const int64_t ngb = (B + plan.sub_group - 1) / plan.sub_group + 1;
@@ -2868,7 +3031,7 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
         t += buf((size_t)nz * 2 * PLANE_FFT_L * sizeof(float2));
     t += buf((size_t)nfft_max * sizeof(float2)) + buf(need_series) + buf(need_sums) + 3 * buf(need_fft) +
          buf(need_plane) + buf((size_t)total_taps * sizeof(float2)) + buf((size_t)5 * nz * sizeof(int32_t)) +
-         buf(subu) + buf(bx);
+         buf(subu) + buf(bx) + buf(ddt);
     return t;
 }
 

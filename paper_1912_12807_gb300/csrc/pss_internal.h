@@ -193,6 +193,9 @@ struct Ctx {
     std::vector<int32_t> delays_host;  // what delays_dev holds (keep list + delays), empty if unknown
     uint64_t delays_gen = 0;           // bumped whenever delays_dev is rewritten
     std::shared_ptr<void> path_cache;  // last search set-up (api.cu), valid while delays_gen matches
+    std::shared_ptr<void> dd_cache;    // last set-up of pss_dedisperse / pss_single_pulse, likewise
+    DevBuf xbits;        // rows of bits of a 1-bit file (bit-sliced dedispersion)
+    DevBuf ddtab[2];     // tables of the shared-sum dedispersion: the search path's batches, the plain calls'
     DevBuf series;       // float [B][nfft]
     DevBuf sums;         // unsigned long long [B]
     DevBuf fftA, fftB;   // float2 [B][M]
@@ -354,6 +357,88 @@ bool dedisp_item(DedispItem* it, int chunk_kb, size_t* shm);
 // largest item's.
 cudaError_t launch_dedisp_multi(const DedispItem* items, int nitems, int64_t total_ctas, size_t shm, bool wide,
                                 cudaStream_t s);
+
+// Dedispersion with partial sums shared between the trials of a group
+// (k_dedisp_sh.cu; its tables: host_dedisp.cpp).
+constexpr int DD_TN = 512;             // native samples per tile
+constexpr int DD_GT = 32;              // trials per group
+constexpr int DD_M = 5;                // 4-sample columns that a thread forms at a time (odd: no bank conflicts)
+constexpr int DD_MAXUNITS = 24;        // units per chunk
+constexpr int DD_MAXROWS = 64;         // rows per chunk (whole rounds of the 16 warps that form them)
+constexpr int DD_RAWCAP = 27 * 1024;   // staged channel bytes per chunk
+constexpr int DD_UCAP = 77 * 1024;     // rows of a chunk (16-bit sums)
+struct DdChunk {
+    int32_t c0, nch;        // channels
+    int32_t S, nunit;       // channels per unit, units
+    int32_t nrow, nrun;     // rows, runs of DD_M columns per row
+    int32_t ishift;         // a row's runs take 2^ishift threads: the smallest power of two >= max(nrun, 32)
+    int32_t flush;          // write the sums out after this chunk
+    // in the blob: this record, the next chunk's record and channel entries (int2, 4 per unit at most), the rows'
+    // sources (uint4: per channel (aligned byte offset << 5) | bit shift), the trials' unit
+    // counts (uint16: at even offsets | at odd << 8) and lists (npair words of two 16-bit word offsets each)
+    int32_t src_off, cnt_off, list_off, npair;
+    int32_t blob_bytes, tx_bytes;
+    int64_t blob_off;       // from the tables' start
+};
+static_assert(sizeof(DdChunk) == 64, "a multiple of 16 bytes");
+constexpr int DD_BLOBHEAD = 2 * sizeof(DdChunk) + DD_MAXUNITS * 4 * 8;
+struct DdTables {
+    int ngroups = 0;
+    size_t chunk_off = 0, chan_off = 0;
+    double cost = 0;             // estimated shared-memory accesses (host_dedisp.cpp)
+    std::vector<uint8_t> bytes;  // what the kernel reads
+};
+// Tables of nb trials with delays [nb][ck]; false where a delay spread does
+// not fit the kernel's shared memory.
+bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, DdTables* out);
+// Device bytes the tables of n trials in batches of nb can take at most.
+size_t dd_tables_bound(int64_t n, int64_t ck, int64_t nb);
+struct DdArgs {
+    const uint8_t* xcm;
+    int64_t pitch;
+    int32_t ck;
+    const uint8_t* tab;          // DdTables::bytes on the device (16-byte aligned)
+    size_t chunk_off, chan_off;
+    int32_t nb;
+    int64_t nv;                  // outputs per trial
+    int32_t lds;                 // ds = 2^lds <= DD_TN
+    float* out_f;                // [nb][out_stride] or null
+    int32_t* out_i;              // [nb][out_stride] or null
+    int64_t out_stride;
+    int32_t vec4;                // float rows start on 16-byte boundaries
+    unsigned long long* sums;    // [nb] or null
+    int* err;
+    int32_t wait_polls;
+};
+cudaError_t launch_dedisp_sh(const DdArgs& a, cudaStream_t s);
+
+// Bit-sliced dedispersion of 1-bit files with at most 255 kept channels
+// (k_dedisp_b1.cu).  Rows of bits: channel c at xb + c * pitchb, bit i of its
+// 32-bit word w the sample 32 w + i.
+constexpr int B1_SLACK = 32 * 1024;  // bytes past the last row that a copy may read
+inline int64_t b1_pitch(int64_t nsamp) { return ((nsamp + 4096 + 1024) / 8 + 15) & ~int64_t(15); }
+inline size_t b1_bytes(int64_t ck, int64_t nsamp) { return (size_t)ck * (size_t)b1_pitch(nsamp) + B1_SLACK; }
+struct B1Args {
+    const uint8_t* xb;
+    int64_t pitchb;
+    int32_t ck, ckp, rowb;       // kept channels; padded count and row bytes in shared memory (set by the launch)
+    int32_t G;                   // trials per CTA (a multiple of 16)
+    const int32_t* delays;       // [nb][ck]
+    int32_t nb;
+    int64_t nv;
+    int32_t lds;                 // ds = 2^lds <= 1024
+    float* out_f;                // [nb][out_stride] or null
+    int32_t* out_i;              // [nb][out_stride] or null
+    int64_t out_stride;
+    int32_t vec4;                // float rows start on 16-byte boundaries
+    unsigned long long* sums;    // [nb] or null
+    int* err;
+    int32_t wait_polls;
+};
+// Whether a launch fits: spread = the largest delay spread of G consecutive trials.
+bool b1_sizes(int32_t spread, int32_t ck, int G, int* KW, int* rowb, size_t* shm);
+cudaError_t launch_prep_bits(const PrepArgs& a, uint8_t* xb, int64_t pitchb, cudaStream_t s);
+cudaError_t launch_dedisp_b1(B1Args a, int32_t spread, cudaStream_t s);
 
 // Two-stage scheme, stage 2: s_i[t] = sum_b u_{g(i),b}[t + D_b(i)], then the
 // ds boxcar, for the nb trials of a batch (k_subband.cu).
