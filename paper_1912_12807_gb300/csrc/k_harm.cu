@@ -310,6 +310,134 @@ __global__ void __launch_bounds__(REG_NT) k_harm_reg(const __grid_constant__ Har
     reg_stages<0, NSTAGES, R>(a, P, acc, hw, j, lane, b);
 }
 
+// ---- 2-D planes: tiles of rows ------------------------------------------------
+//
+// A thread owns RT rows at HP half-bins (lanes consecutive in h, 32 apart per
+// point).  The rows of a tile are |j - Z| = RT a + r, r < RT, on one side of
+// the centre row, and n divides RT, so harmonic k of stage n reads row
+//   |j_k - Z| = (RT / n) k a + floor((2 k r + n) / (2 n)):
+// which of the RT points share a row is known when the kernel is compiled, and
+// each distinct row is loaded once (8 harmonics, 8 rows: 40 loads per half-bin
+// instead of 64; 16 harmonics, 16 rows: 139 instead of 256).  The additions are
+// those of the kernels above in the same order, so the sums are bit-identical.
+// Bound: the latency of plane reads that miss L2 (a plane of 201 rows is larger
+// than L2; 1.5 planes come from HBM, 3.3 from L2).  301 trials, 201 rows of
+// 2^18, 8 harmonics: 27.6 ms with one row per warp, 22.0 ms here; 1, 2 and 4
+// half-bins per thread 31.2, 23.1 and 22.0 ms (longer contiguous reads and more
+// of them in flight), 256 threads per block 22.3 ms.
+template <int NSTAGES>
+struct TileRows {
+    static constexpr int value = NSTAGES <= 4 ? 8 : 16;
+};
+
+// The rare path: a warp with points of row j at or above the threshold.
+template <int SI, int HP>
+__device__ __noinline__ void tile_hit(const HarmArgs& a, const float* P, float4 v, int hw, int j, int lane, int b) {
+    static_assert(HP <= 4, "points by value");
+    const float w[4] = {v.x, v.y, v.z, v.w};
+    float acc[HP];
+#pragma unroll
+    for (int i = 0; i < HP; ++i) acc[i] = w[i];
+    reg_test<SI, HP>(a, P, acc, hw, j, lane, b);
+}
+
+template <int SI, int NSTAGES, int RT, int HP>
+__device__ __forceinline__ void tile_stages(const HarmArgs& a, const char* Pz, int rstep, int ta, float (&acc)[RT][HP],
+                                            int hw, int nrow, int sgn, int d0, int lane, int b) {
+    if constexpr (SI < NSTAGES) {
+        constexpr int n = 1 << SI;
+        if constexpr (SI > 0) {
+#pragma unroll
+            for (int q = 0; q < n / 2; ++q) {
+                const int k = 2 * q + 1;
+                // (rows of the last tile past the plane's edge are loaded from the edge row and not tested)
+                const int row0 = (RT / n) * k * ta;
+                const int hb = 4 * ((2 * k * (hw + lane) + n) >> (SI + 1));
+                float v[HP];
+#pragma unroll
+                for (int r = 0; r < RT; ++r) {
+                    const int c = (2 * k * r + n) / (2 * n);
+                    if (r == 0 || c != (2 * k * (r - 1) + n) / (2 * n)) {
+                        const char* p = Pz + (int64_t)(min(row0 + c, a.Z) * rstep) + hb;
+#pragma unroll
+                        for (int i = 0; i < HP; ++i) v[i] = __ldg(reinterpret_cast<const float*>(p) + (32 / n) * k * i);
+                    }
+#pragma unroll
+                    for (int i = 0; i < HP; ++i) acc[r][i] += v[i];
+                }
+            }
+        }
+        float mx = acc[0][0];
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+#pragma unroll
+            for (int i = 0; i < HP; ++i) mx = fmaxf(mx, acc[r][i]);
+        if (__any_sync(0xffffffffu, mx >= a.thr[SI])) {
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                float m = acc[r][0];
+#pragma unroll
+                for (int i = 1; i < HP; ++i) m = fmaxf(m, acc[r][i]);
+                // (the centre row belongs to the side d >= 0)
+                if (r < nrow && (r > 0 || d0 > 0 || sgn > 0) && __any_sync(0xffffffffu, m >= a.thr[SI]))
+                    tile_hit<SI, HP>(a, a.plane + (int64_t)b * a.plane_stride, 
+                                     make_float4(acc[r][0], acc[r][HP > 1 ? 1 : 0], acc[r][HP > 2 ? 2 : 0], acc[r][HP > 3 ? 3 : 0]), hw,
+                                     a.Z + sgn * (d0 + r), lane, b);
+            }
+        }
+        tile_stages<SI + 1, NSTAGES, RT, HP>(a, Pz, rstep, ta, acc, hw, nrow, sgn, d0, lane, b);
+    }
+}
+
+constexpr int TILE_HP = 4;
+constexpr int TILE_NT = 128;
+
+template <int NSTAGES>
+__global__ void __launch_bounds__(TILE_NT) k_harm_tile(const __grid_constant__ HarmArgs a) {
+    constexpr int RT = TileRows<NSTAGES>::value, HP = TILE_HP;
+    const int lane = threadIdx.x & 31;
+    // row tiles fastest: the harmonic rows that successive blocks read overlap while they are in L2
+    const int sgn = (blockIdx.x & 1) ? -1 : 1, ta = blockIdx.x >> 1, d0 = RT * ta;
+    const int b = blockIdx.z;
+    const int hw = (blockIdx.y * (TILE_NT / 32) + (threadIdx.x >> 5)) * 32 * HP;
+    const int nrow = min(RT, a.Z + 1 - d0);  // rows of the tile inside the plane
+    const int rstep = sgn * (int)a.nfft * 4;
+    const char* Pz = reinterpret_cast<const char*>(a.plane + (int64_t)b * a.plane_stride + (int64_t)a.Z * a.nfft);
+    float acc[RT][HP];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+        const char* p = Pz + (int64_t)(min(d0 + r, a.Z) * rstep) + 4 * (hw + lane);
+#pragma unroll
+        for (int i = 0; i < HP; ++i) acc[r][i] = __ldg(reinterpret_cast<const float*>(p) + 32 * i);
+    }
+    tile_stages<0, NSTAGES, RT, HP>(a, Pz, rstep, ta, acc, hw, nrow, sgn, d0, lane, b);
+}
+
+// Planes with rows on both sides of the centre row, offsets within 31 bits of bytes from it, whole warps.
+bool tile_usable(const HarmArgs& a) {
+    return a.nz > 1 && a.nz == 2 * a.Z + 1 && a.nstages <= 5 && (int64_t)(a.Z + 16) * a.nfft * 4 < (int64_t(1) << 31) &&
+           a.nfft % (TILE_NT * TILE_HP) == 0 && a.nfft / (TILE_NT * TILE_HP) <= 65535 && a.nb <= 65535;
+}
+
+template <int NSTAGES>
+cudaError_t launch_tile_t(const HarmArgs& a, cudaStream_t s) {
+    constexpr int RT = TileRows<NSTAGES>::value;
+    dim3 grid((unsigned)(2 * ((a.Z + RT) / RT)), (unsigned)(a.nfft / (TILE_NT * TILE_HP)), (unsigned)a.nb);
+    k_harm_tile<NSTAGES><<<grid, TILE_NT, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tile(const HarmArgs& a, cudaStream_t s) {
+    switch (a.nstages) {
+        case 1: return launch_tile_t<1>(a, s);
+        case 2: return launch_tile_t<2>(a, s);
+        case 3: return launch_tile_t<3>(a, s);
+        case 4: return launch_tile_t<4>(a, s);
+        case 5: return launch_tile_t<5>(a, s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 // 2-D planes: the warps of a block take consecutive plane rows (default; 31.1 -> 28.9 ms on
 // the zmax 200 accel file); PSS_HARM_ROWS=0 keeps one row per block
 bool harm_rows() {
@@ -348,6 +476,7 @@ cudaError_t launch_reg(const HarmArgs& a, cudaStream_t s) {
 cudaError_t launch_harm(const HarmArgs& a, cudaStream_t s) {
     if (a.nfft > (int64_t(1) << 24) || a.nstages > 6) return cudaErrorInvalidValue;
     if ((int64_t)a.nz * a.nfft > (int64_t(1) << 31)) return cudaErrorInvalidValue;  // 32-bit plane offsets
+    if (harm_rows() && tile_usable(a)) return launch_tile(a, s);
     // register-blocked kernel: up to 16 harmonics, whole warps of 32 x 16 points
     if (a.run == 8 && a.nstages <= 5 && a.nfft % (REG_NT * 8) == 0 && a.nfft / (REG_NT * 8) <= 65535 &&
         a.nb <= 65535)
