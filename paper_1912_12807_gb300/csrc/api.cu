@@ -291,16 +291,6 @@ pss_status enqueue_prep(pss_ctx* ctx, const pss_fil_desc* fil, const uint8_t* sr
     return PSS_OK;
 }
 
-// Old entry used by pss_dedisperse: set-up, upload and unpack in one go.
-pss_status stage_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, const void* data,
-                       int on_device, int64_t dm_begin, int64_t dm_end, cudaStream_t s, int32_t* ck_out,
-                       int64_t* pitch_out, SubTab* T) {
-    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, ck_out, pitch_out, T));
-    const uint8_t* src = nullptr;
-    PSS_TRY(upload_input(ctx, fil, data, on_device, s, &src));
-    return enqueue_prep(ctx, fil, src, *ck_out, *pitch_out, s);
-}
-
 // max over the dedispersion kernel's groups of consecutive trials and over
 // channels of (dmax - dmin)
 int32_t delay_spread(const int32_t* d, int64_t nb, int32_t ck, int G = dedisp_group_trials()) {
@@ -432,7 +422,8 @@ pss_status dd_upload(pss_ctx* ctx, int which, const std::vector<uint8_t>& host, 
 pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_t pitch, const SubTab& T,
                           const StageInfo& st, int64_t dm_begin, int64_t b0, int32_t nb, int32_t spread,
                           const SubBatch& SB, const DdBatch& dd, void* subu, float* out_f,
-                          int32_t* out_i, int64_t out_stride, unsigned long long* sums, cudaStream_t s) {
+                          int32_t* out_i, int64_t out_stride, unsigned long long* sums, cudaStream_t s,
+                          unsigned long long* squares = nullptr) {
     const int32_t* base = (const int32_t*)ctx->delays_dev.p;
     if (!T.on && dd.kind == DD_BITS) {
         B1Args ba{};
@@ -449,6 +440,7 @@ pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_
         ba.out_stride = out_stride;
         ba.vec4 = out_f && out_stride % 4 == 0 && ((uintptr_t)out_f & 15) == 0;
         ba.sums = sums;
+        ba.squares = squares;
         ba.err = (int*)ctx->errflag.p;
         ba.wait_polls = ctx->wait_polls;
         ProfScope ps(ctx, 1, s);
@@ -506,6 +498,7 @@ pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_
         da.out_stride = out_stride;
         da.vec4 = out_f && out_stride % 4 == 0 && ((uintptr_t)out_f & 15) == 0;
         da.sums = sums;
+        da.squares = squares;
         da.err = (int*)ctx->errflag.p;
         da.wait_polls = ctx->wait_polls;
         ProfScope ps(ctx, 1, s);
@@ -585,15 +578,18 @@ pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_
 // detection kernel); per trial, the detections by S/N (descending; ties:
 // smaller width, then earlier) are kept when their interval [t, t + w)
 // overlaps none kept before.  Output sorted by (trial, t).
-void sp_prune(std::vector<SpRaw>& raw, const std::vector<unsigned long long>& mom, int64_t dm_begin, int64_t dm_end,
+void sp_prune(const std::vector<SpRaw>& raw, const std::vector<unsigned long long>& mom, int64_t dm_begin, int64_t dm_end,
               const pss_plan* plan, std::vector<pss_sp_event>* out) {
-    std::sort(raw.begin(), raw.end(), [](const SpRaw& a, const SpRaw& b) {
-        return a.dm_idx != b.dm_idx ? a.dm_idx < b.dm_idx : (a.w != b.w ? a.w < b.w : a.t < b.t);
-    });
+    // detections by trial (a counting sort; the order within a trial does not matter: they are sorted by S/N below)
     const int64_t nt = dm_end - dm_begin;
-    std::vector<size_t> start(nt + 1, raw.size());
-    for (size_t i = raw.size(); i-- > 0;) start[raw[i].dm_idx - dm_begin] = i;
-    for (int64_t i = nt - 1; i >= 0; --i) start[i] = std::min(start[i], start[i + 1]);
+    std::vector<size_t> start(nt + 1, 0);
+    for (const SpRaw& e : raw) ++start[e.dm_idx - dm_begin + 1];
+    for (int64_t i = 0; i < nt; ++i) start[i + 1] += start[i];
+    std::vector<SpRaw> by(raw.size());
+    {
+        std::vector<size_t> at(start.begin(), start.end() - 1);
+        for (const SpRaw& e : raw) by[at[e.dm_idx - dm_begin]++] = e;
+    }
     std::vector<std::vector<pss_sp_event>> per(nt);
     parallel_for_fn(nt, 8, [&](int64_t i) {
         const size_t a = start[i], b = start[i + 1];
@@ -607,12 +603,12 @@ void sp_prune(std::vector<SpRaw>& raw, const std::vector<unsigned long long>& mo
         std::vector<pss_sp_event> ev;
         for (size_t k = a; k < b; ++k) {
             pss_sp_event e;
-            e.dm_idx = raw[k].dm_idx;
-            e.width = raw[k].w;
-            e.t = raw[k].t;
-            e.boxsum = raw[k].B;
-            const double w = (double)raw[k].w;
-            e.snr = ((double)raw[k].B - w * mu) / (sigma * sqrt(w));
+            e.dm_idx = by[k].dm_idx;
+            e.width = by[k].w;
+            e.t = by[k].t;
+            e.boxsum = by[k].B;
+            const double w = (double)by[k].w;
+            e.snr = ((double)by[k].B - w * mu) / (sigma * sqrt(w));
             ev.push_back(e);
         }
         std::sort(ev.begin(), ev.end(), [](const pss_sp_event& x, const pss_sp_event& y) {
@@ -870,8 +866,10 @@ std::string path_key(const pss_plan* plan, const pss_fil_desc* fil, const pss_se
 // Host set-up of a plain dedispersion (pss_dedisperse, pss_single_pulse) of
 // [dm_begin, dm_end): input tables, DM batches, shared-sum tables and the
 // stage-1 buffer, kept like PathCache while the request is the same and the
-// device tables are still the ones uploaded for it.
-enum DdUse { DD_DEDISPERSE, DD_SINGLE_PULSE };
+// device tables are still the ones uploaded for it.  pss_fold keeps the input
+// tables of the whole plan (its trials change from call to call), which are
+// those of a search of the whole plan.
+enum DdUse { DD_DEDISPERSE, DD_SINGLE_PULSE, DD_FOLD };
 
 struct DdSetup {
     std::string key;
@@ -882,6 +880,8 @@ struct DdSetup {
     std::vector<BatchDesc> batches;  // out_off: samples of the trials before, packed
     size_t need_subu = 0;
     bool need_bytes = false, need_bits = false;
+    std::vector<int32_t> keep;       // pss_fold: the kept channels
+    DdBatch fold;                    // pss_fold: how its runs of trials are dedispersed
 };
 
 pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin, int64_t dm_end,
@@ -889,7 +889,8 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     const pss_search_cfg none{};
     std::string key = path_key(plan, fil, &none, dm_begin, dm_end, MODE_SPECTRUM, (int64_t)use, 0, ctx->tune);
     key_put(&key, ctx->tune.bx_min);
-    auto kept = std::static_pointer_cast<DdSetup>(ctx->dd_cache);
+    std::shared_ptr<void>& slot = use == DD_FOLD ? ctx->fold_cache : ctx->dd_cache;
+    auto kept = std::static_pointer_cast<DdSetup>(slot);
     if (kept && kept->key == key && dm_end > dm_begin) {
         if (kept->gen != ctx->delays_gen) {  // another request's delays are on the device
             SubTab T;
@@ -903,6 +904,30 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     auto D = std::make_shared<DdSetup>();
     PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T));
     D->need_bytes = D->T.on;
+    if (use == DD_FOLD) {
+        // bit-sliced where any 16 consecutive trials' delays fit (delays are monotonic in DM)
+        D->keep = kept_channels(fil);
+        int32_t spread = 0;
+        for (const auto& st : plan->stages)
+            for (int64_t i = st.first; i + 1 < st.first + st.n_dm; ++i) {
+                const int64_t e = std::min<int64_t>(i + 15, st.first + st.n_dm - 1);
+                for (int32_t c : D->keep)
+                    spread = std::max(spread, std::abs(plan->delays[(size_t)e * plan->nchan + c] - plan->delays[(size_t)i * plan->nchan + c]));
+            }
+        int KW, rowb;
+        size_t shm;
+        if (fil->nbits == 1 && !D->T.on && b1_sizes(spread, D->ck, 16, &KW, &rowb, &shm)) {
+            D->fold.kind = DD_BITS;
+            D->fold.group = 16;
+            D->fold.spread = spread;
+        }
+        (D->fold.kind == DD_BITS ? D->need_bits : D->need_bytes) = true;
+        D->key.swap(key);
+        D->gen = ctx->delays_gen;
+        slot = D;
+        *out = D;
+        return PSS_OK;
+    }
     const std::vector<int32_t> hd = D->T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
     std::vector<uint8_t> dd_host;
     int64_t off = 0;
@@ -940,7 +965,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     PSS_TRY(dd_upload(ctx, 1, dd_host, s));
     D->key.swap(key);
     D->gen = ctx->delays_gen;
-    ctx->dd_cache = D;
+    slot = D;
     *out = D;
     return PSS_OK;
 }
@@ -2112,11 +2137,13 @@ pss_status pss_single_pulse(pss_ctx* ctx, const pss_plan* plan, const pss_fil_de
             PSS_TRY(ctx->sp_series.ensure((size_t)nb * st.nv * sizeof(int32_t)));
             PSS_TRY(ctx->sp_mom.ensure((size_t)(2 + SP_MAXW) * nb * sizeof(unsigned long long)));
             int32_t* ser = (int32_t*)ctx->sp_series.p;
-            PSS_TRY(enqueue_dedisp(ctx, plan, D->ck, D->pitch, D->T, st, dm_begin, b0, nb, d.spread, d.sub, d.dd,
-                                   ctx->subu.p, nullptr, ser, st.nv, nullptr, s));
             unsigned long long* m1 = (unsigned long long*)ctx->sp_mom.p;
             unsigned long long* m2 = m1 + nb;
             PSS_CUDA(cudaMemsetAsync(m1, 0, (size_t)2 * nb * sizeof(unsigned long long), s));
+            // the shared-sum and bit-sliced kernels form the moments with the series
+            const bool mom = !D->T.on && d.dd.kind != DD_DIRECT;
+            PSS_TRY(enqueue_dedisp(ctx, plan, D->ck, D->pitch, D->T, st, dm_begin, b0, nb, d.spread, d.sub, d.dd,
+                                   ctx->subu.p, nullptr, ser, st.nv, mom ? m1 : nullptr, s, mom ? m2 : nullptr));
             PSS_CUDA(cudaMemsetAsync(ctx->counter.p, 0, sizeof(unsigned long long), s));
             SpArgs sa{};
             sa.series = ser;
@@ -2136,7 +2163,7 @@ pss_status pss_single_pulse(pss_ctx* ctx, const pss_plan* plan, const pss_fil_de
             sa.out = (SpRaw*)ctx->sp_ev.p;
             sa.count = (unsigned long long*)ctx->counter.p;
             sa.cap = devcap;
-            PSS_CUDA(launch_single_pulse(sa, m1, m2, s));
+            PSS_CUDA(launch_single_pulse(sa, m1, m2, mom, s));
             unsigned long long cnt = 0;
             PSS_CUDA(cudaMemcpyAsync(&cnt, ctx->counter.p, sizeof(cnt), cudaMemcpyDeviceToHost, s));
             PSS_CUDA(cudaStreamSynchronize(s));
@@ -2199,11 +2226,12 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
     PSS_TRY(check_common(ctx, plan, fil, data, lo_dm, hi_dm + 1));
     PSS_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t s = pick_stream(ctx, stream);
-    int32_t ck = 0;
-    int64_t pitch = 0;
-    SubTab T;
-    PSS_TRY(stage_input(ctx, plan, fil, data, data_on_device, lo_dm, hi_dm + 1, s, &ck, &pitch, &T));
-    const std::vector<int32_t> hd = T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), lo_dm, hi_dm + 1);
+    std::shared_ptr<DdSetup> D;
+    PSS_TRY(setup_dedisp(ctx, plan, fil, 0, plan->ndm(), DD_FOLD, s, &D));
+    const int32_t ck = D->ck;
+    const uint8_t* src = nullptr;
+    PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
+    PSS_TRY(enqueue_prep(ctx, fil, src, ck, D->pitch, s, D->need_bytes, D->need_bits));
     // requests by trial; chunks of at most 256 series rows
     std::vector<int64_t> order(n);
     for (int64_t i = 0; i < n; ++i) order[i] = i;
@@ -2244,17 +2272,17 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
             const int32_t nb = (int32_t)(r.b - r.a);
             int32_t spread = 0;
             SubBatch SB;
-            if (T.on) {
-                SB = sub_batch(plan, T, ck, lo_dm, r.a, nb, st.nv, st.ds);
+            if (D->T.on) {
+                SB = sub_batch(plan, D->T, ck, 0, r.a, nb, st.nv, st.ds);
                 PSS_TRY(ctx->subu.ensure((size_t)plan->nsub * SB.ngb * SB.stride1 * 4 + subsum_slack_bytes(SB.spread2)));
-            } else {
-                spread = delay_spread(hd.data() + (size_t)(r.a - lo_dm) * ck, nb, ck);
+            } else if (D->fold.kind == DD_DIRECT) {
+                spread = delay_spread(compact_delays(plan, D->keep, r.a, r.b).data(), nb, ck);
             }
             int32_t* out = ser + (int64_t)r.row0 * nv_max;
-            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, lo_dm, r.a, nb, spread, SB, DdBatch(),
-                                   ctx->subu.p, nullptr, out,
-                                   nv_max, nullptr, s));
-            PSS_CUDA(launch_sp_moments(out, nv_max, st.nv, nb, m1 + r.row0, m2 + r.row0, s));
+            const bool mom = D->fold.kind == DD_BITS;  // the bit-sliced kernel forms the moments with the series
+            PSS_TRY(enqueue_dedisp(ctx, plan, ck, D->pitch, D->T, st, 0, r.a, nb, spread, SB, D->fold, ctx->subu.p, nullptr,
+                                   out, nv_max, mom ? m1 + r.row0 : nullptr, s, mom ? m2 + r.row0 : nullptr));
+            if (!mom) PSS_CUDA(launch_sp_moments(out, nv_max, st.nv, nb, m1 + r.row0, m2 + r.row0, s));
         }
         std::vector<unsigned long long> mom((size_t)2 * MAXROWS);
         PSS_CUDA(cudaMemcpyAsync(mom.data(), m1, mom.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
@@ -2294,6 +2322,9 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
         fa.items = (const FoldItem*)(fb + o_items);
         fa.nbin = nbin;
         fa.nfreq = nfreq;
+        int32_t ds_max = 1;
+        for (const Run& r : runs) ds_max = std::max(ds_max, plan->stages[plan->stage_of[r.a]].ds);
+        fa.max_value = (long long)ck * (fil->nbits == 8 ? 255 : 1) * ds_max;
         fa.step_bins = step_bins;
         fa.prof = (long long*)(fb + o_prof);
         fa.counts = (long long*)(fb + o_cnt);

@@ -121,15 +121,18 @@ __device__ __forceinline__ void planes_to_bytes(uint32_t (&p)[8], uint32_t (&n)[
     }
 }
 
-// Bytes of 1024 consecutive samples (sl) summed by ds and written from output j.
+// Bytes of 1024 consecutive samples (sl) summed by ds and written from output j; their sum, and the squares added
+// to m2 (integer rows with a.squares).
 template <bool INT_OUT>
-__device__ __forceinline__ uint32_t put_bytes(const B1Args& a, const uint32_t* sl, int my, int64_t j, int lane) {
+__device__ __forceinline__ uint32_t put_bytes(const B1Args& a, const uint32_t* sl, int my, int64_t j, int lane,
+                                              unsigned long long& m2) {
     const int ds = 1 << a.lds;
     int32_t* o = (INT_OUT ? a.out_i : reinterpret_cast<int32_t*>(a.out_f)) + (int64_t)my * a.out_stride + j;
     const int left = (int)min((int64_t)(SLICE >> a.lds), a.nv - j);
     uint32_t part = 0;
     auto store = [&](int q, uint32_t v) {
         part += v;
+        if (INT_OUT && a.squares) m2 += (unsigned long long)v * v;
         if (INT_OUT) o[q] = (int32_t)v;
         else reinterpret_cast<float*>(o)[q] = (float)v;
     };
@@ -260,7 +263,7 @@ __global__ void __launch_bounds__(NT, 2) k_dedisp_b1(const __grid_constant__ B1A
                 }
             }
         }
-        unsigned long long part = 0ull;
+        unsigned long long part = 0ull, m2 = 0ull;
 #pragma unroll
         for (int k = 0; k < KW; ++k) {
             const int64_t t = t0 + 1024 * k;
@@ -273,12 +276,17 @@ __global__ void __launch_bounds__(NT, 2) k_dedisp_b1(const __grid_constant__ B1A
             reinterpret_cast<uint4*>(sl)[2 * lane] = make_uint4(n[0], n[1], n[2], n[3]);
             reinterpret_cast<uint4*>(sl)[2 * lane + 1] = make_uint4(n[4], n[5], n[6], n[7]);
             __syncwarp();
-            part += put_bytes<INT_OUT>(a, sl, g0 + tr, j, lane);
+            part += put_bytes<INT_OUT>(a, sl, g0 + tr, j, lane, m2);
         }
         if (a.sums) {
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
             if (lane == 0) atomicAdd(a.sums + g0 + tr, part);
+        }
+        if (INT_OUT && a.squares) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, off);
+            if (lane == 0) atomicAdd(a.squares + g0 + tr, m2);
         }
     }
 }

@@ -144,38 +144,62 @@ struct Acc {
 
 // One trial's tile out: ds native samples to an output, 32-bit integers added
 // to what an earlier flush of this tile left (`prev`), converted on the last.
+// Adds the outputs and their squares to m1 and m2 (integer rows with a.squares: the moments of the single-pulse search).
 template <bool INT_OUT>
-__device__ __forceinline__ unsigned long long put(const DdArgs& a, const uint32_t* nat, int my, int64_t t0, int lane,
-                                                  bool prev, bool last) {
+__device__ __forceinline__ void put(const DdArgs& a, const uint32_t* nat, int my, int64_t t0, int lane, bool prev, bool last,
+                                    unsigned long long& m1, unsigned long long& m2) {
     const int64_t j0 = t0 >> a.lds;
     int32_t* o = (INT_OUT ? a.out_i : reinterpret_cast<int32_t*>(a.out_f)) + (int64_t)my * a.out_stride + j0;
     const int left = (int)min((int64_t)(TN >> a.lds), a.nv - j0);  // outputs of this tile
-    unsigned long long part = 0ull;
     if (a.lds == 0 && !prev && last && left == TN && (INT_OUT || a.vec4)) {
         if (INT_OUT) {
+            uint32_t sum = 0;
 #pragma unroll
-            for (int i = 0; i < TN / 32; ++i) o[lane + 32 * i] = (int32_t)nat[lane + 32 * i];
-            return 0ull;
+            for (int i = 0; i < TN / 32; ++i) {
+                const uint32_t v = nat[lane + 32 * i];
+                o[lane + 32 * i] = (int32_t)v;
+                if (a.squares) {
+                    sum += v;  // 16 values of at most 65535
+                    m2 += (unsigned long long)v * v;
+                }
+            }
+            m1 += sum;
+            return;
         }
-        uint32_t sum = 0;  // 16 values of at most 65535
+        uint32_t sum = 0;
 #pragma unroll
         for (int i = 0; i < TN / 128; ++i) {
             const uint4 v = reinterpret_cast<const uint4*>(nat)[lane + 32 * i];
             sum += v.x + v.y + v.z + v.w;
             reinterpret_cast<float4*>(o)[lane + 32 * i] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
         }
-        return sum;
+        m1 += sum;
+        return;
     }
     const int ds = 1 << a.lds;
     for (int q = lane; q < left; q += 32) {
         uint32_t v = 0;
         for (int e = 0; e < ds; ++e) v += nat[(q << a.lds) + e];
         if (prev) v += (uint32_t)o[q];
-        if (last) part += v;
+        if (last) {
+            m1 += v;
+            if (INT_OUT && a.squares) m2 += (unsigned long long)v * v;
+        }
         if (INT_OUT || !last) o[q] = (int32_t)v;
         else reinterpret_cast<float*>(o)[q] = (float)v;
     }
-    return part;
+}
+
+// The warp's moments of trial `my` added to the trial's.
+__device__ __forceinline__ void add_moments(const DdArgs& a, int my, int lane, unsigned long long m1, unsigned long long m2) {
+    if (!a.sums) return;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m1 += __shfl_xor_sync(0xffffffffu, m1, off);
+    if (lane == 0) atomicAdd(a.sums + my, m1);
+    if (!a.squares) return;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, off);
+    if (lane == 0) atomicAdd(a.squares + my, m2);
 }
 
 template <bool INT_OUT>
@@ -248,26 +272,20 @@ __global__ void __launch_bounds__(NT, 2) k_dedisp_sh(const __grid_constant__ DdA
             const bool last = c + 1 == gi.y;
             __syncthreads();
             uint32_t* nat = u + warp * TN;
-            unsigned long long p0 = 0ull, p1 = 0ull;
             if (act0) {
+                unsigned long long m1 = 0ull, m2 = 0ull;
                 A0.write(nat, lane);
                 __syncwarp();
-                p0 = put<INT_OUT>(a, nat, g * GT + warp, t0, lane, prev, last);
+                put<INT_OUT>(a, nat, g * GT + warp, t0, lane, prev, last, m1, m2);
+                if (last) add_moments(a, g * GT + warp, lane, m1, m2);
                 __syncwarp();
             }
             if (act1) {
+                unsigned long long m1 = 0ull, m2 = 0ull;
                 A1.write(nat, lane);
                 __syncwarp();
-                p1 = put<INT_OUT>(a, nat, g * GT + warp + NW, t0, lane, prev, last);
-            }
-            if (last && a.sums) {
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    p0 += __shfl_xor_sync(0xffffffffu, p0, off);
-                    p1 += __shfl_xor_sync(0xffffffffu, p1, off);
-                }
-                if (lane == 0 && act0) atomicAdd(a.sums + g * GT + warp, p0);
-                if (lane == 0 && act1) atomicAdd(a.sums + g * GT + warp + NW, p1);
+                put<INT_OUT>(a, nat, g * GT + warp + NW, t0, lane, prev, last, m1, m2);
+                if (last) add_moments(a, g * GT + warp + NW, lane, m1, m2);
             }
             A0.clear();
             A1.clear();

@@ -194,6 +194,7 @@ struct Ctx {
     uint64_t delays_gen = 0;           // bumped whenever delays_dev is rewritten
     std::shared_ptr<void> path_cache;  // last search set-up (api.cu), valid while delays_gen matches
     std::shared_ptr<void> dd_cache;    // last set-up of pss_dedisperse / pss_single_pulse, likewise
+    std::shared_ptr<void> fold_cache;  // last set-up of pss_fold, likewise
     DevBuf xbits;        // rows of bits of a 1-bit file (bit-sliced dedispersion)
     DevBuf ddtab[2];     // tables of the shared-sum dedispersion: the search path's batches, the plain calls'
     DevBuf series;       // float [B][nfft]
@@ -406,7 +407,8 @@ struct DdArgs {
     int32_t* out_i;              // [nb][out_stride] or null
     int64_t out_stride;
     int32_t vec4;                // float rows start on 16-byte boundaries
-    unsigned long long* sums;    // [nb] or null
+    unsigned long long* sums;    // [nb] sum of the series, or null
+    unsigned long long* squares; // [nb] sum of its squares (integer rows), or null
     int* err;
     int32_t wait_polls;
 };
@@ -431,7 +433,8 @@ struct B1Args {
     int32_t* out_i;              // [nb][out_stride] or null
     int64_t out_stride;
     int32_t vec4;                // float rows start on 16-byte boundaries
-    unsigned long long* sums;    // [nb] or null
+    unsigned long long* sums;    // [nb] sum of the series, or null
+    unsigned long long* squares; // [nb] sum of its squares (integer rows), or null
     int* err;
     int32_t wait_polls;
 };
@@ -540,8 +543,9 @@ struct SpArgs {
     unsigned long long* count;
     int64_t cap;
 };
-// moments (into s1, s2, which must be zeroed) then detection
-cudaError_t launch_single_pulse(const SpArgs& a, unsigned long long* s1, unsigned long long* s2, cudaStream_t s);
+// moments (into s1, s2, which must be zeroed; have_moments: they are there already) then detection
+cudaError_t launch_single_pulse(const SpArgs& a, unsigned long long* s1, unsigned long long* s2, bool have_moments,
+                                cudaStream_t s);
 // detection alone (moments already in a.s1, a.s2)
 cudaError_t launch_sp_detect_only(const SpArgs& a, cudaStream_t s);
 // exact moments alone: s1[b] += sum s, s2[b] += sum s^2 (zero them first)
@@ -562,6 +566,7 @@ struct FoldArgs {
     int64_t stride;
     const FoldItem* items;
     int32_t nbin, nfreq;
+    long long max_value;    // largest value a series sample can take (0: unknown)
     double step_bins;
     long long* prof;        // [items][nfreq][nbin]
     long long* counts;      // [items][nfreq][nbin]
