@@ -257,6 +257,7 @@ class Plan:
     def __init__(self, desc: FilDesc, stages, subband=None):
         self.desc = desc
         self._st = stages_array(stages)
+        self._lengths = None
         h = C.c_void_p()
         if subband is None:
             _check(lib().pss_dd_plan(C.byref(desc.c), self._st, len(stages), C.byref(h)))
@@ -297,6 +298,17 @@ class Plan:
         _check(lib().pss_plan_trial_info(self.h, int(dm_idx), C.byref(s), C.byref(nv), C.byref(nfft), C.byref(ds)))
         return dict(stage=s.value, nv=nv.value, nfft=nfft.value, ds=ds.value)
 
+    def stage_lengths(self):
+        """[(trials, trial info of the first of them)] of the plan's non-empty stages."""
+        if self._lengths is None:
+            out, first = [], 0
+            for st in self._st:
+                if st.n_dm > 0:
+                    out.append((st.n_dm, self.trial(first)))
+                    first += st.n_dm
+            self._lengths = out
+        return self._lengths
+
     def close(self):
         if self.h:
             lib().pss_plan_free(self.h)
@@ -335,8 +347,15 @@ def _stream(stream):
     return None
 
 
-def _rows(plan: Plan, dm_begin: int, dm_end: int, key: str):
-    return [plan.trial(i)[key] for i in range(dm_begin, dm_end)]
+def _total(plan: Plan, dm_begin: int, dm_end: int, key: str, per: int = 1) -> int:
+    """Sum of a trial length (nv or nfft, divided by `per`) over the trials [dm_begin, dm_end): a
+    stage's trials have the same lengths.  A range outside the plan counts what is inside; the
+    library call that follows refuses it."""
+    total, first = 0, 0
+    for n, t in plan.stage_lengths():
+        total += max(0, min(dm_end, first + n) - max(dm_begin, first)) * (t[key] // per)
+        first += n
+    return total
 
 
 # ---------------------------------------------------------------------------
@@ -346,7 +365,7 @@ def _rows(plan: Plan, dm_begin: int, dm_end: int, key: str):
 def pss_dedisperse(ctx: Context, plan: Plan, data, dm_begin: int, dm_end: int, out=None, stream=None):
     """int32 device tensor of the packed dedispersed series of [dm_begin, dm_end)."""
     import torch
-    total = int(sum(_rows(plan, dm_begin, dm_end, "nv")))
+    total = _total(plan, dm_begin, dm_end, "nv")
     if out is None:
         out = torch.empty(max(total, 1), dtype=torch.int32, device="cuda:%d" % ctx.device)
     p, dev, keep = _data_arg(data)
@@ -360,7 +379,7 @@ def pss_dedisperse_noalloc(plan: Plan, data_dev, dm_begin: int, dm_end: int, out
     a CUDA tensor, `out` (allocated here if not given, before the call) an
     int32 CUDA tensor of at least sum N_v elements."""
     import torch
-    total = int(sum(_rows(plan, dm_begin, dm_end, "nv")))
+    total = _total(plan, dm_begin, dm_end, "nv")
     if out is None:
         out = torch.empty(max(total, 1), dtype=torch.int32, device=data_dev.device)
     if not (isinstance(data_dev, torch.Tensor) and data_dev.is_cuda):
@@ -411,7 +430,7 @@ def pss_fold(ctx: Context, plan: Plan, data, dm_idx, f_hz, fdot_hz_s=None, nbin:
 def pss_spectrum(ctx: Context, plan: Plan, data, cfg: pss_search_cfg, dm_begin: int, dm_end: int, stream=None):
     """complex64 device tensor: whitened half spectra, rows packed back to back."""
     import torch
-    total = int(sum(n // 2 for n in _rows(plan, dm_begin, dm_end, "nfft")))
+    total = _total(plan, dm_begin, dm_end, "nfft", 2)
     out = torch.empty(2 * max(total, 1), dtype=torch.float32, device="cuda:%d" % ctx.device)
     p, dev, keep = _data_arg(data)
     _check(lib().pss_spectrum(ctx.h, plan.h, C.byref(plan.desc.c), p, dev, C.byref(cfg), dm_begin, dm_end,
@@ -427,7 +446,7 @@ def pss_power_plane(ctx: Context, plan: Plan, data, cfg: pss_search_cfg, dm_begi
     """float32 device tensor: planes [n_z][nfft] of [dm_begin, dm_end) packed back to back."""
     import torch
     nz = n_z(cfg)
-    total = int(sum(nz * n for n in _rows(plan, dm_begin, dm_end, "nfft")))
+    total = nz * _total(plan, dm_begin, dm_end, "nfft")
     out = torch.empty(max(total, 1), dtype=torch.float32, device="cuda:%d" % ctx.device)
     p, dev, keep = _data_arg(data)
     _check(lib().pss_power_plane(ctx.h, plan.h, C.byref(plan.desc.c), p, dev, C.byref(cfg), dm_begin, dm_end,
