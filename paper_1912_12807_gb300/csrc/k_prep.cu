@@ -53,14 +53,17 @@ __device__ __forceinline__ void prep_tile(const PrepArgs& a, int64_t bx, int by)
 
 __global__ void __launch_bounds__(256) k_prep(PrepArgs a) { prep_tile(a, blockIdx.x, blockIdx.y); }
 
-// 8-bit time-major file with every channel kept (row r = channel r): thread
-// (group g of 4 channels, run of 16 samples) reads the run's 16 words of its
-// 4 channels (a warp: 32 consecutive groups, 128 contiguous bytes per
-// sample), transposes each 4 x 4 block of bytes with byte permutes, and
-// writes 16 samples of each of its channels as one 16-byte store.  The 8
-// warps of a CTA take 8 consecutive runs.
+// 8-bit time-major file: thread (group g of 4 channels, run of 16 samples)
+// reads the run's 16 words of its 4 channels (a warp: 32 consecutive groups,
+// 128 contiguous bytes per sample), transposes each 4 x 4 block of bytes with
+// byte permutes, and writes 16 samples of each of its channels as one 16-byte
+// store.  The 8 warps of a CTA take 8 consecutive runs.  ALL: every channel is
+// kept (row r = channel r); else a channel's row is its place in the keep list
+// (increasing), and channels that are not in it are not written: 400 channels
+// x 200 003 samples, 57 masked, 139 us with the tiled kernel, 51 us here.
 constexpr int U8RUN = 16;
 
+template <bool ALL>
 __global__ void __launch_bounds__(256) k_prep_u8(const PrepArgs a) {
     const int ng = a.nchan >> 2;
     const int g = (int)blockIdx.y * 32 + (int)(threadIdx.x & 31);
@@ -85,10 +88,23 @@ __global__ void __launch_bounds__(256) k_prep_u8(const PrepArgs a) {
         o[2][q] = __byte_perm(hi01, hi23, 0x5410);
         o[3][q] = __byte_perm(hi01, hi23, 0x7632);
     }
+    int r = 4 * g;
+    if (!ALL) {
+        // first kept row at or after channel 4 g
+        int lo = 0, hi = a.ck;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (__ldg(a.keep + mid) < 4 * g) lo = mid + 1;
+            else hi = mid;
+        }
+        r = lo;
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<uint4*>(a.xcm + (int64_t)(4 * g + i) * a.pitch + t0) =
-            make_uint4(o[i][0], o[i][1], o[i][2], o[i][3]);
+    for (int i = 0; i < 4; ++i) {
+        if (!ALL && (r >= a.ck || __ldg(a.keep + r) != 4 * g + i)) continue;
+        *reinterpret_cast<uint4*>(a.xcm + (int64_t)r * a.pitch + t0) = make_uint4(o[i][0], o[i][1], o[i][2], o[i][3]);
+        ++r;
+    }
 }
 
 // 1-bit time-major file with every channel kept: a warp takes 32
@@ -165,14 +181,15 @@ cudaError_t launch_prep_multi(const PrepItem* items, int nitems, int64_t total_c
 }
 
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t s) {
-    // every channel kept, file order: row r is channel r
-    const bool all = a.ck == a.nchan && a.layout == 0 && prep_fast() && (a.pitch & 63) == 0;
-    if (all && a.nbits == 8 && (a.nchan & 3) == 0 && ((uintptr_t)a.src & 3) == 0) {
+    // file order; every channel kept: row r is channel r
+    const bool file = a.layout == 0 && prep_fast() && (a.pitch & 63) == 0, all = a.ck == a.nchan;
+    if (file && a.nbits == 8 && (a.nchan & 3) == 0 && ((uintptr_t)a.src & 3) == 0) {
         dim3 g8((unsigned)((a.pitch + 8 * U8RUN - 1) / (8 * U8RUN)), (unsigned)((a.nchan / 4 + 31) / 32));
-        k_prep_u8<<<g8, 256, 0, s>>>(a);
+        if (all) k_prep_u8<true><<<g8, 256, 0, s>>>(a);
+        else k_prep_u8<false><<<g8, 256, 0, s>>>(a);
         return cudaGetLastError();
     }
-    if (all && a.nbits == 1 && (a.nchan & 7) == 0) {
+    if (file && all && a.nbits == 1 && (a.nchan & 7) == 0) {
         k_prep_u1<<<(unsigned)((a.pitch + 255) / 256), 256, 0, s>>>(a);
         return cudaGetLastError();
     }
