@@ -426,7 +426,6 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
 // sub-stages (radix 16, 16, 8) instead of four: fewer shared-memory passes
 // and barriers per row, at lower thread count.
 constexpr int F16NT = 128;
-constexpr int F16CTAS = 4;          // CTAs per SM
 constexpr int T16A = 0;             // RR 16, NS 16: 16 x 16
 constexpr int T16B = T16A + 256;    // RR 8, NS 256: 8 x 256
 constexpr int T16N = T16B + 2048;
@@ -474,7 +473,7 @@ __device__ __forceinline__ void fft2048x2_r16(float2* b0, float2* b1, const floa
     fft16_substage2<8, 256>(b0, b1, twt + T16B);
 }
 
-__global__ void __launch_bounds__(F16NT, F16CTAS) k_plane_fft16(const __grid_constant__ PlaneArgs a, int rows_per) {
+__global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant__ PlaneArgs a) {
     constexpr int L = PLANE_FFT_L;
     constexpr int NE = L / F16NT;  // 16 bins per thread
     extern __shared__ float2 fsm[];
@@ -505,14 +504,14 @@ __global__ void __launch_bounds__(F16NT, F16CTAS) k_plane_fft16(const __grid_con
 #pragma unroll
     for (int e = 0; e < NE; ++e) X[e] = Y0[fx(threadIdx.x + e * F16NT)];
     __syncthreads();
-    const int r_lo = blockIdx.z * rows_per, r_hi = min(a.nz, r_lo + rows_per);
+    const int nz = a.nz;
     float2* P = reinterpret_cast<float2*>(a.plane + (int64_t)b * a.plane_stride);
     // Per row: the first radix-16 sub-stage (running span 1) takes butterfly b = thread's
     // elements b + 128 q, which are the thread's own bins X[q]: it runs on the products in
     // registers; the middle sub-stage runs in shared memory; the last (radix 8, span 256)
     // reads its inputs and writes the powers of its outputs b + 256 q straight to the plane.
     // The same operations in the same order as the in-place form (bit-identical output).
-    for (int j = r_lo; j < r_hi; ++j) {
+    for (int j = 0; j < nz; ++j) {
         const bool zrow0 = (j == a.zrow0);
         const float2* T0 = a.ftaps + (int64_t)j * 2 * L;
         const float2* T1 = T0 + L;
@@ -612,22 +611,8 @@ cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s) {
         const size_t shm = (size_t)(2 * PLANE_FFT_L + T16N) * sizeof(float2);
         cudaError_t e = allow_smem((const void*)k_plane_fft16, shm);
         if (e != cudaSuccess) return e;
-        // Every CTA takes the same time, so a last wave that is half empty costs a whole one: the rows are split over
-        // gridDim.z where that shortens the waves (a CTA's set-up counts as two rows).  301 trials x 201 rows of 2^18
-        // in batches of 29 (3.5 waves of 608 CTAs): 37.7 ms unsplit, 36.9 ms with half the rows each.
-        const int64_t ctas = (M + a.fV - 1) / a.fV * a.nb, slots = (int64_t)(a.num_sms > 0 ? a.num_sms : 152) * F16CTAS;
-        int rows_per = a.nz;
-        double best = 1e300;
-        for (int split = 1; split <= 8 && split <= a.nz; ++split) {
-            const int rows = (a.nz + split - 1) / split;
-            const double t = (double)((ctas * ((a.nz + rows - 1) / rows) + slots - 1) / slots) * (rows + 2.0);
-            if (t < 0.99 * best) {
-                best = t;
-                rows_per = rows;
-            }
-        }
-        dim3 grid((unsigned)((M + a.fV - 1) / a.fV), (unsigned)a.nb, (unsigned)((a.nz + rows_per - 1) / rows_per));
-        k_plane_fft16<<<grid, F16NT, shm, s>>>(a, rows_per);
+        dim3 grid((unsigned)((M + a.fV - 1) / a.fV), (unsigned)a.nb);
+        k_plane_fft16<<<grid, F16NT, shm, s>>>(a);
         return cudaGetLastError();
     }
     if (a.ftaps) {
