@@ -283,7 +283,8 @@ __global__ void k_fft_templates(FftTemplateArgs a) {
         __syncthreads();
     }
     const double scale = 1.0 / ((double)a.L * sqrt(red[0]));
-    float2* out = a.ftaps + (int64_t)blockIdx.x * a.L;
+    // row's spectra of both parities interleaved: (re 0, re 1, im 0, im 1) per bin
+    float* out = reinterpret_cast<float*>(a.ftaps + (int64_t)row * 2 * a.L) + par;
     for (int f = threadIdx.x; f < a.L; f += blockDim.x) {
         double re = 0.0, im = 0.0;
         for (int i = 0; i < 2 * m; ++i) {
@@ -292,7 +293,8 @@ __global__ void k_fft_templates(FftTemplateArgs a) {
             re += g[i].x * w.x - g[i].y * w.y;
             im += g[i].x * w.y + g[i].y * w.x;
         }
-        out[f] = make_float2((float)(re * scale), (float)(im * scale));
+        out[4 * f] = (float)(re * scale);
+        out[4 * f + 2] = (float)(im * scale);
     }
 }
 
@@ -390,12 +392,12 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
     float2* P = reinterpret_cast<float2*>(a.plane + (int64_t)b * a.plane_stride);
     for (int j = 0; j < nz; ++j) {
         const bool zrow0 = (j == a.zrow0);
-        const float2* T0 = a.ftaps + (int64_t)j * 2 * L;
-        const float2* T1 = T0 + L;
+        const float4* T = reinterpret_cast<const float4*>(a.ftaps + (int64_t)j * 2 * L);
 #pragma unroll
         for (int e = 0; e < NE; ++e) {
             const int i = threadIdx.x + e * FNT;
-            const float2 y0 = cmul(X[e], __ldg(T0 + i)), y1 = cmul(X[e], __ldg(T1 + i));
+            const float4 t = __ldg(T + i);
+            const float2 y0 = cmul(X[e], make_float2(t.x, t.z)), y1 = cmul(X[e], make_float2(t.y, t.w));
             Y0[fp(i)] = make_float2(y0.x, -y0.y);
             Y1[fp(i)] = make_float2(y1.x, -y1.y);
         }
@@ -421,65 +423,138 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
     }
 }
 
-// ---- overlap-save plane, radix 16-16-8 form (an autotuner choice) -------------------
-// The same correlation as k_plane_fft with 128 threads and three in-place
-// sub-stages (radix 16, 16, 8) instead of four: fewer shared-memory passes
-// and barriers per row, at lower thread count.
+// ---- overlap-save plane, radix 16-16-8 form ------------------------------------------
+// The same correlation as k_plane_fft with 128 threads and three sub-stages
+// (radix 16, 16, 8).  The transforms of the two parities have the same
+// twiddles, so they are carried as pairs (re 0, re 1), (im 0, im 1) and every
+// addition and multiplication is one packed instruction on both
+// (add / mul / fma .f32x2); an element of both is 16 bytes in shared memory.
+//
+// Per row, the first sub-stage (running span 1) takes butterfly b = the
+// thread's own segment bins b + 128 q times the template spectra, in
+// registers; the middle one runs in shared memory; the last (radix 8, span
+// 256) reads its inputs and writes the powers of its outputs b + 256 q
+// straight to the plane.
+//
+// Bound by the chain load - butterfly - barrier of a row with 16 warps per SM
+// (registers), not by a unit: leaving out the template loads, the
+// twiddles, the arithmetic or the stores saves 5 to 16 % each.  So the first
+// F16PRE template quads of the next row are loaded before the last sub-stage.
+// 301 trials x 201 rows of 2^18 (with the harmonic sums and the rest of the
+// search): 62.3 ms with scalar arithmetic, 61.5 packed, 61.25 with 4 quads
+// loaded ahead (8: 62.8, spills); 8 trials x 201 rows of 2^18 (plane call):
+// 1203 -> 1192 -> 1181 us.
 constexpr int F16NT = 128;
+constexpr int F16PRE = 4;           // template quads of the next row loaded ahead
 constexpr int T16A = 0;             // RR 16, NS 16: 16 x 16
 constexpr int T16B = T16A + 256;    // RR 8, NS 256: 8 x 256
 constexpr int T16N = T16B + 2048;
 
-template <int RR, int NS>
-__device__ __forceinline__ void fft16_substage2(float2* b0, float2* b1, const float2* twt) {
-    constexpr int L = PLANE_FFT_L;
-    constexpr int NB = L / RR;
-    constexpr int PER = NB / F16NT;
-    float2 x0[PER][RR], x1[PER][RR];
-    int dst[PER];
+struct cc {  // a complex number of each parity
+    float2 re, im;
+};
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ cc cadd(cc a, cc b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
+__device__ __forceinline__ cc csub(cc a, cc b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
+// both parities times one complex number w (cmul's roundings)
+__device__ __forceinline__ cc cmul1(cc a, float wr, float wi) {
+    const float2 r = make_float2(wr, wr), i = make_float2(wi, wi), ni = make_float2(-wi, -wi);
+    return {fma2(a.re, r, mul2(a.im, ni)), fma2(a.re, i, mul2(a.im, r))};
+}
+__device__ __forceinline__ void dft4(cc& y0, cc& y1, cc& y2, cc& y3) {
+    const cc s02 = cadd(y0, y2), d02 = csub(y0, y2), s13 = cadd(y1, y3), d = csub(y1, y3);
+    y0 = cadd(s02, s13);
+    y2 = csub(s02, s13);
+    // d02 +- (-i) d
+    y1 = {add2(d02.re, d.im), sub2(d02.im, d.re)};
+    y3 = {sub2(d02.re, d.im), add2(d02.im, d.re)};
+}
+__device__ __forceinline__ void dft8(cc (&x)[8]) {
+    cc a0 = cadd(x[0], x[4]), b0 = csub(x[0], x[4]);
+    cc a1 = cadd(x[1], x[5]), b1 = csub(x[1], x[5]);
+    cc a2 = cadd(x[2], x[6]), b2 = csub(x[2], x[6]);
+    cc a3 = cadd(x[3], x[7]), b3 = csub(x[3], x[7]);
+    const float2 h = make_float2(R2, R2), nh = make_float2(-R2, -R2);
+    b1 = {mul2(add2(b1.re, b1.im), h), mul2(sub2(b1.im, b1.re), h)};
+    b2 = {b2.im, mul2(b2.re, make_float2(-1.f, -1.f))};
+    b3 = {mul2(sub2(b3.im, b3.re), h), mul2(add2(b3.re, b3.im), nh)};
+    dft4(a0, a1, a2, a3);
+    dft4(b0, b1, b2, b3);
+    x[0] = a0; x[2] = a1; x[4] = a2; x[6] = a3;
+    x[1] = b0; x[3] = b1; x[5] = b2; x[7] = b3;
+}
+__device__ __forceinline__ void dft16(cc (&x)[16]) {
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-        const int b = threadIdx.x + p * F16NT;
-        const int k = b & (NS - 1);
+    for (int n2 = 0; n2 < 4; ++n2) {
+        dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);
 #pragma unroll
-        for (int q = 0; q < RR; ++q) {
-            x0[p][q] = b0[fx(b + q * NB)];
-            x1[p][q] = b1[fx(b + q * NB)];
-            if (NS > 1 && q) {
-                const float2 w = twt[q * NS + k];
-                x0[p][q] = cmul(x0[p][q], w);
-                x1[p][q] = cmul(x1[p][q], w);
+        for (int k1 = 1; k1 < 4; ++k1)
+            if (n2) {
+                const float2 w = w16(n2 * k1);
+                if (n2 * k1 == 4) x[4 * k1 + n2] = {x[4 * k1 + n2].im, mul2(x[4 * k1 + n2].re, make_float2(-1.f, -1.f))};
+                else x[4 * k1 + n2] = cmul1(x[4 * k1 + n2], w.x, w.y);
             }
+    }
+    cc y[16];
+#pragma unroll
+    for (int k1 = 0; k1 < 4; ++k1) {
+        dft4(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) y[k1 + 4 * k2] = x[4 * k1 + k2];
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = y[i];
+}
+// Shared-memory slot of element i (16 bytes): within a run of 8 the slot is XORed with the run of 16's number,
+// so that the strided writes of the first sub-stage and the consecutive accesses hit 8 different bank groups.
+__device__ __forceinline__ int fs(int i) { return i ^ ((i >> 4) & 7); }
+__device__ __forceinline__ cc ldc(const float4* b, int i) {
+    const float4 v = b[fs(i)];
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ void stc(float4* b, int i, cc x) { b[fs(i)] = make_float4(x.re.x, x.re.y, x.im.x, x.im.y); }
+
+// The middle sub-stage, radix 16, running span 16, in place.
+__device__ __forceinline__ void mid16(float4* Y, const float2* twt) {
+    const int b = threadIdx.x, k = b & 15;
+    cc x[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+        x[q] = ldc(Y, b + q * 128);
+        if (q) {
+            const float2 w = twt[q * 16 + k];
+            x[q] = cmul1(x[q], w.x, w.y);
         }
-        dst[p] = (b - k) * RR + k;
     }
     __syncthreads();
+    dft16(x);
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-        dft_any<RR>(x0[p]);
-        dft_any<RR>(x1[p]);
-#pragma unroll
-        for (int q = 0; q < RR; ++q) {
-            b0[fx(dst[p] + q * NS)] = x0[p][q];
-            b1[fx(dst[p] + q * NS)] = x1[p][q];
-        }
-    }
+    for (int q = 0; q < 16; ++q) stc(Y, (b - k) * 16 + k + q * 16, x[q]);
     __syncthreads();
 }
 
-__device__ __forceinline__ void fft2048x2_r16(float2* b0, float2* b1, const float2* twt) {
-    fft16_substage2<16, 1>(b0, b1, twt);
-    fft16_substage2<16, 16>(b0, b1, twt + T16A);
-    fft16_substage2<8, 256>(b0, b1, twt + T16B);
+// Inputs of butterfly bb of the last sub-stage, radix 8, running span 256, transformed.
+__device__ __forceinline__ void last8(const float4* Y, const float2* tl, int bb, cc (&x)[8]) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        x[q] = ldc(Y, bb + q * 256);
+        if (q) {
+            const float2 w = tl[q * 256 + bb];
+            x[q] = cmul1(x[q], w.x, w.y);
+        }
+    }
+    dft8(x);
 }
 
 __global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant__ PlaneArgs a) {
     constexpr int L = PLANE_FFT_L;
     constexpr int NE = L / F16NT;  // 16 bins per thread
-    extern __shared__ float2 fsm[];
-    float2* Y0 = fsm;
-    float2* Y1 = fsm + L;
-    float2* twt = fsm + 2 * L;
+    extern __shared__ float4 f16sm[];
+    float4* Y = f16sm;
+    float2* twt = reinterpret_cast<float2*>(Y + L);
     const int b = blockIdx.y;
     const int64_t M = a.nfft / 2;
     const int V = a.fV, M0 = a.fM0;
@@ -493,83 +568,81 @@ __global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant_
         const int q = o / ns, k = o - q * ns;
         twt[i] = a.tw[(int64_t)(q * k * (L / (rr * ns))) * tstride];
     }
-    for (int i = threadIdx.x; i < L; i += F16NT) {
-        const int64_t k = k0 - M0 + i;
-        Y0[fx(i)] = (k >= 0 && k < M) ? Ap[k] : make_float2(0.f, 0.f);
-        Y1[fx(i)] = make_float2(0.f, 0.f);
+    // the segment's spectrum (the second parity idle); each thread keeps the bins it multiplies
+    float2 X[NE];
+    {
+        cc x[NE];
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int64_t k = k0 - M0 + threadIdx.x + e * F16NT;
+            const float2 v = (k >= 0 && k < M) ? Ap[k] : make_float2(0.f, 0.f);
+            x[e] = {make_float2(v.x, 0.f), make_float2(v.y, 0.f)};
+        }
+        dft16(x);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) stc(Y, threadIdx.x * 16 + q, x[q]);
     }
     __syncthreads();
-    fft2048x2_r16(Y0, Y1, twt);
-    float2 X[NE];
+    mid16(Y, twt + T16A);
+    {
+        cc z[2][8];
+        last8(Y, twt + T16B, threadIdx.x, z[0]);
+        last8(Y, twt + T16B, threadIdx.x + F16NT, z[1]);
+        // outputs b + 256 q of butterflies tid and tid + 128: the bins tid + 128 e
 #pragma unroll
-    for (int e = 0; e < NE; ++e) X[e] = Y0[fx(threadIdx.x + e * F16NT)];
+        for (int q = 0; q < 8; ++q) {
+            X[2 * q] = make_float2(z[0][q].re.x, z[0][q].im.x);
+            X[2 * q + 1] = make_float2(z[1][q].re.x, z[1][q].im.x);
+        }
+    }
     __syncthreads();
     const int nz = a.nz;
     float2* P = reinterpret_cast<float2*>(a.plane + (int64_t)b * a.plane_stride);
-    // Per row: the first radix-16 sub-stage (running span 1) takes butterfly b = thread's
-    // elements b + 128 q, which are the thread's own bins X[q]: it runs on the products in
-    // registers; the middle sub-stage runs in shared memory; the last (radix 8, span 256)
-    // reads its inputs and writes the powers of its outputs b + 256 q straight to the plane.
-    // The same operations in the same order as the in-place form (bit-identical output).
+    float4 tp[F16PRE];
+#pragma unroll
+    for (int e = 0; e < F16PRE; ++e) tp[e] = __ldg(reinterpret_cast<const float4*>(a.ftaps) + threadIdx.x + e * F16NT);
     for (int j = 0; j < nz; ++j) {
         const bool zrow0 = (j == a.zrow0);
-        const float2* T0 = a.ftaps + (int64_t)j * 2 * L;
-        const float2* T1 = T0 + L;
+        const float4* T = reinterpret_cast<const float4*>(a.ftaps + (int64_t)j * 2 * L) + threadIdx.x;
         {
-            float2 x0[NE], x1[NE];
+            cc x[NE];
 #pragma unroll
             for (int e = 0; e < NE; ++e) {
-                const int i = threadIdx.x + e * F16NT;
-                const float2 y0 = cmul(X[e], __ldg(T0 + i)), y1 = cmul(X[e], __ldg(T1 + i));
-                x0[e] = make_float2(y0.x, -y0.y);
-                x1[e] = make_float2(y1.x, -y1.y);
+                // conj(X T) of both parities
+                const float4 t = e < F16PRE ? tp[e < F16PRE ? e : 0] : __ldg(T + e * F16NT);
+                const float2 tr = make_float2(t.x, t.y), ti = make_float2(t.z, t.w);
+                const float2 xr = make_float2(X[e].x, X[e].x), nxr = make_float2(-X[e].x, -X[e].x);
+                const float2 nxi = make_float2(-X[e].y, -X[e].y);
+                x[e] = {fma2(xr, tr, mul2(nxi, ti)), fma2(nxr, ti, mul2(nxi, tr))};
             }
-            dft_any<16>(x0);
-            dft_any<16>(x1);
+            dft16(x);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                Y0[fx(threadIdx.x * 16 + q)] = x0[q];
-                Y1[fx(threadIdx.x * 16 + q)] = x1[q];
-            }
+            for (int q = 0; q < 16; ++q) stc(Y, threadIdx.x * 16 + q, x[q]);
         }
         __syncthreads();
-        fft16_substage2<16, 16>(Y0, Y1, twt + T16A);
-        float2* row = P + (int64_t)j * M;
-        {
-            constexpr int NS = 256, NB = L / 8, PER = NB / F16NT;
-            const float2* tl = twt + T16B;
+        mid16(Y, twt + T16A);
+        if (j + 1 < nz) {
 #pragma unroll
-            for (int p = 0; p < PER; ++p) {
-                const int bb = threadIdx.x + p * F16NT;  // < NS: its span index k is bb itself
-                float2 x0[8], x1[8];
+            for (int e = 0; e < F16PRE; ++e) tp[e] = __ldg(T + 2048 + e * F16NT);
+        }
+        float2* row = P + (int64_t)j * M + k0;
+        const int left = (int)min((int64_t)V, M - k0);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    x0[q] = Y0[fx(bb + q * NB)];
-                    x1[q] = Y1[fx(bb + q * NB)];
-                    if (q) {
-                        const float2 w = tl[q * NS + bb];
-                        x0[q] = cmul(x0[q], w);
-                        x1[q] = cmul(x1[q], w);
-                    }
-                }
-                dft_any<8>(x0);
-                dft_any<8>(x1);
+        for (int p = 0; p < 2; ++p) {
+            const int bb = threadIdx.x + p * F16NT;
+            cc x[8];
+            last8(Y, twt + T16B, bb, x);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int u = bb + q * NS;
-                    const int64_t k = k0 + u;
-                    if (u < V && k < M) {
-                        float p0 = pow2(x0[q]);
-                        if (zrow0) {
-                            const float2 c = Ap[k];
-                            p0 = pow2(c);
-                        }
-                        row[k] = make_float2(p0, pow2(x1[q]));
-                    }
+            for (int q = 0; q < 8; ++q) {
+                const int u = bb + q * 256;
+                if (u < left) {
+                    float2 pw = fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re));
+                    if (zrow0) pw.x = pow2(Ap[k0 + u]);  // integer half-bins of the z = 0 row: the raw powers, exactly
+                    row[u] = pw;
                 }
             }
         }
-        __syncthreads();  // the next row's first sub-stage overwrites Y0 / Y1
+        __syncthreads();  // the next row's first sub-stage overwrites Y
     }
 }
 
@@ -608,7 +681,7 @@ cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s) {
     const int nz = a.zmax ? (int)llround(2.0 * a.zmax / a.dz) + 1 : 1;
     if (a.ftaps && a.form == 1) {
         if (a.fL != PLANE_FFT_L || a.fV <= 0 || a.twM % PLANE_FFT_L) return cudaErrorInvalidValue;
-        const size_t shm = (size_t)(2 * PLANE_FFT_L + T16N) * sizeof(float2);
+        const size_t shm = (size_t)PLANE_FFT_L * sizeof(float4) + T16N * sizeof(float2);
         cudaError_t e = allow_smem((const void*)k_plane_fft16, shm);
         if (e != cudaSuccess) return e;
         dim3 grid((unsigned)((M + a.fV - 1) / a.fV), (unsigned)a.nb);

@@ -205,7 +205,7 @@ struct Ctx {
     DevBuf cands;        // pss_raw_cand [cap]
     DevBuf counter;      // unsigned long long
     DevBuf taps;         // float2 templates
-    DevBuf ftaps;        // float2 [nz][2][L] template spectra (overlap-save plane)
+    DevBuf ftaps;        // float4 [nz][L] template spectra of both parities (overlap-save plane)
     DevBuf tapinfo;      // per row tap info
     DevBuf errflag;      // int: a kernel's bounded wait expired
     DevBuf twid;         // float2 twiddle table exp(-2 pi i t / twid_n)
@@ -646,8 +646,8 @@ struct PlaneArgs {
     const int32_t* tap_off;  // [nz*2] offsets into taps
     const int32_t* tap_m;    // [nz] half-widths
     const float* tap_scale;  // [nz*2] 1/sqrt(E)
-    // overlap-save form (zmax > 0): per (row, parity) the spectrum of the
-    // taps, [nz][2][fL]; null when the direct form is used
+    // overlap-save form (zmax > 0): per row the spectra of both parities' taps,
+    // [nz][fL] of (re 0, re 1, im 0, im 1); null when the direct form is used
     const float2* ftaps;
     int32_t fL, fV, fM0;     // segment length, valid outputs per segment, lead
     int32_t nz, zrow0;       // rows, and the row with z = 0 exactly (-1: none)
@@ -668,7 +668,7 @@ struct FftTemplateArgs {
     int32_t nz, zmax, extra;
     double dz;
     const int32_t* tap_m;  // [nz] half-widths
-    float2* ftaps;         // out [nz][2][L]
+    float2* ftaps;         // out [nz][L] of (re 0, re 1, im 0, im 1)
     int32_t L, M0;
 };
 cudaError_t launch_fft_templates(const FftTemplateArgs& a, cudaStream_t s);
