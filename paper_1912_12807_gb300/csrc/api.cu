@@ -196,12 +196,38 @@ void subband_tables(const pss_plan* plan, const std::vector<int32_t>& keep, int6
     T->e_host.assign(h + T->e_off, h + T->e_off + ng * ck);
 }
 
+// Room for the boxcar table of the downsampled rows of [dm_begin, dm_end) (exact plans only).
+pss_status ensure_bx(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_t dm_begin, int64_t dm_end) {
+    if (plan->nsub > 0) return PSS_OK;
+    size_t need_bx = 0;
+    for (const auto& st : plan->stages)
+        if (st.n_dm > 0 && st.first < dm_end && st.first + st.n_dm > dm_begin && bx_use(ctx->tune, st.ds) && ck <= 65535)
+            need_bx = std::max(need_bx, bx_table_bytes(ck, plan->nsamp, st.ds));
+    if (need_bx) {
+        const void* was = ctx->bx.p;
+        PSS_TRY(ctx->bx.ensure(need_bx));
+        if (ctx->bx.p != was) ctx->bx_ds = 0;
+    }
+    return PSS_OK;
+}
+
 // Host-side set-up for a file: the kept channels, their delays for
 // [dm_begin, dm_end) (or the two-stage tables, `T`) uploaded to
 // ctx->delays_dev, and the channel-major buffer.  Synchronises `s` (the
 // delay upload reads a host vector).
 pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin,
-                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr) {
+                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr,
+                       bool bx = true) {
+    // a call that fails part-way may have replaced the tables or given up a buffer: set-ups kept for them end
+    struct Done {
+        pss_ctx* ctx;
+        bool ok = false;
+        ~Done() {
+            if (ok) return;
+            ctx->delays_host.clear();
+            ctx->delays_gen++;
+        }
+    } done{ctx};
     const std::vector<int32_t> keep = kept_channels(fil);
     const int32_t ck = (int32_t)keep.size();
     if (ck == 0) return fail(PSS_EINVAL, "channel mask removes every channel");
@@ -229,19 +255,7 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
     }
     PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
     if (fil->nbits == 1 && plan->nsub == 0 && ck <= 255) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
-    // the boxcar table of the downsampled rows (exact plans only)
-    if (plan->nsub == 0) {
-        size_t need_bx = 0;
-        for (const auto& st : plan->stages)
-            if (st.n_dm > 0 && st.first < dm_end && st.first + st.n_dm > dm_begin && bx_use(ctx->tune, st.ds) &&
-                ck <= 65535)
-                need_bx = std::max(need_bx, bx_table_bytes(ck, plan->nsamp, st.ds));
-        if (need_bx) {
-            const void* was = ctx->bx.p;
-            PSS_TRY(ctx->bx.ensure(need_bx));
-            if (ctx->bx.p != was) ctx->bx_ds = 0;
-        }
-    }
+    if (bx) PSS_TRY(ensure_bx(ctx, plan, ck, dm_begin, dm_end));
     if (!ctx->errflag.p) {
         PSS_TRY(ctx->errflag.ensure(sizeof(int)));
         PSS_CUDA(cudaMemsetAsync(ctx->errflag.p, 0, sizeof(int), s));
@@ -251,6 +265,7 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
         ctx->delays_host.swap(host);
         ctx->delays_gen++;
     }
+    done.ok = true;
     *ck_out = ck;
     *pitch_out = pitch;
     return PSS_OK;
@@ -678,6 +693,7 @@ pss_status ensure_templates(pss_ctx* ctx, const pss_search_cfg* cfg, cudaStream_
         off[2 * j + 1] = total;
         total += 2 * m[j];
     }
+    ctx->tap_zmax = -1;  // (until the new ones stand)
     PSS_TRY(ctx->taps.ensure((size_t)total * sizeof(float2)));
     PSS_TRY(ctx->tapinfo.ensure((size_t)(2 * nz + nz + 2 * nz) * sizeof(int32_t)));
     int32_t* info = (int32_t*)ctx->tapinfo.p;
@@ -894,7 +910,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     if (kept && kept->key == key && dm_end > dm_begin) {
         if (kept->gen != ctx->delays_gen) {  // another request's delays are on the device
             SubTab T;
-            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &kept->ck, &kept->pitch, &T));
+            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &kept->ck, &kept->pitch, &T, use != DD_FOLD));
             kept->gen = ctx->delays_gen;
         }
         if (kept->need_subu) PSS_TRY(ctx->subu.ensure(kept->need_subu));
@@ -902,7 +918,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
         return PSS_OK;
     }
     auto D = std::make_shared<DdSetup>();
-    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T));
+    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T, use != DD_FOLD));
     D->need_bytes = D->T.on;
     if (use == DD_FOLD) {
         // bit-sliced where any 16 consecutive trials' delays fit (delays are monotonic in DM)
@@ -975,8 +991,13 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
                       int64_t max_b = 0) {
     std::string key = path_key(plan, fil, cfg, dm_begin, dm_end, mode, dev_cap, max_b, ctx->tune);
     PathCache* pc = static_cast<PathCache*>(ctx->path_cache.get());
-    const bool hit = pc && pc->gen == ctx->delays_gen && pc->key == key && dm_end > dm_begin;
+    const bool hit = pc && pc->key == key && dm_end > dm_begin;
     if (hit) {
+        if (pc->gen != ctx->delays_gen) {  // another request's delays are on the device; the rest still stands
+            SubTab T;
+            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &pc->P.ck, &pc->P.pitch, &T));
+            pc->gen = ctx->delays_gen;
+        }
         *P = pc->P;
     } else {
         PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &P->ck, &P->pitch, &P->sub));
@@ -1003,6 +1024,7 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
     int64_t nfft_max = 0;
     for (const auto& st : plan->stages) nfft_max = std::max<int64_t>(nfft_max, st.nfft);
     if (ctx->twid_n < nfft_max) {
+        ctx->twid_n = 0;  // (a refused allocation leaves no table)
         PSS_TRY(ctx->twid.ensure((size_t)nfft_max * sizeof(float2)));
         PSS_CUDA(launch_twiddles((float2*)ctx->twid.p, nfft_max, s));
         ctx->twid_n = nfft_max;
@@ -1783,6 +1805,7 @@ pss_status multi_search(pss_ctx* ctx, const pss_search_cfg* cfg, const pss_multi
     int64_t nfft_max = 0;
     for (const MultiBatch& b : M.batches) nfft_max = std::max(nfft_max, b.nfft);
     if (ctx->twid_n < nfft_max) {
+        ctx->twid_n = 0;  // (a refused allocation leaves no table)
         PSS_TRY(ctx->twid.ensure((size_t)nfft_max * sizeof(float2)));
         PSS_CUDA(launch_twiddles((float2*)ctx->twid.p, nfft_max, s));
         ctx->twid_n = nfft_max;
@@ -2228,6 +2251,7 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
     cudaStream_t s = pick_stream(ctx, stream);
     std::shared_ptr<DdSetup> D;
     PSS_TRY(setup_dedisp(ctx, plan, fil, 0, plan->ndm(), DD_FOLD, s, &D));
+    PSS_TRY(ensure_bx(ctx, plan, D->ck, lo_dm, hi_dm + 1));  // of the rows folded from only
     const int32_t ck = D->ck;
     const uint8_t* src = nullptr;
     PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
