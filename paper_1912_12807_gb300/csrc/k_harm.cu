@@ -318,18 +318,13 @@ __global__ void __launch_bounds__(REG_NT) k_harm_reg(const __grid_constant__ Har
 //   |j_k - Z| = (RT / n) k a + floor((2 k r + n) / (2 n)):
 // which of the RT points share a row is known when the kernel is compiled, and
 // each distinct row is loaded once (8 harmonics, 8 rows: 40 loads per half-bin
-// instead of 64; 16 harmonics, 16 rows: 139 instead of 256).  The additions are
-// those of the kernels above in the same order, so the sums are bit-identical.
+// instead of 64).  The additions are those of the kernels above in the same
+// order, so the sums are bit-identical.
 // Bound: the latency of plane reads that miss L2 (a plane of 201 rows is larger
 // than L2; 1.5 planes come from HBM, 3.3 from L2).  301 trials, 201 rows of
 // 2^18, 8 harmonics: 27.6 ms with one row per warp, 22.0 ms here; 1, 2 and 4
 // half-bins per thread 31.2, 23.1 and 22.0 ms (longer contiguous reads and more
 // of them in flight), 256 threads per block 22.3 ms.
-template <int NSTAGES>
-struct TileRows {
-    static constexpr int value = NSTAGES <= 4 ? 8 : 16;
-};
-
 // The rare path: a warp with points of row j at or above the threshold.
 template <int SI, int HP>
 __device__ __noinline__ void tile_hit(const HarmArgs& a, const float* P, float4 v, int hw, int j, int lane, int b) {
@@ -389,12 +384,13 @@ __device__ __forceinline__ void tile_stages(const HarmArgs& a, const char* Pz, i
     }
 }
 
+constexpr int TILE_RT = 8;  // rows of a tile: a multiple of every stage's number of harmonics
 constexpr int TILE_HP = 4;
 constexpr int TILE_NT = 128;
 
 template <int NSTAGES>
 __global__ void __launch_bounds__(TILE_NT) k_harm_tile(const __grid_constant__ HarmArgs a) {
-    constexpr int RT = TileRows<NSTAGES>::value, HP = TILE_HP;
+    constexpr int RT = TILE_RT, HP = TILE_HP;
     const int lane = threadIdx.x & 31;
     // row tiles fastest: the harmonic rows that successive blocks read overlap while they are in L2
     const int sgn = (blockIdx.x & 1) ? -1 : 1, ta = blockIdx.x >> 1, d0 = RT * ta;
@@ -413,16 +409,25 @@ __global__ void __launch_bounds__(TILE_NT) k_harm_tile(const __grid_constant__ H
     tile_stages<0, NSTAGES, RT, HP>(a, Pz, rstep, ta, acc, hw, nrow, sgn, d0, lane, b);
 }
 
-// Planes with rows on both sides of the centre row, offsets within 31 bits of bytes from it, whole warps.
+// Planes with rows on both sides of the centre row, offsets within 31 bits of bytes from it, whole warps, up to 8
+// harmonics (16 would need tiles of 16 rows, 64 sums per thread).
 bool tile_usable(const HarmArgs& a) {
-    return a.nz > 1 && a.nz == 2 * a.Z + 1 && a.nstages <= 5 && (int64_t)(a.Z + 16) * a.nfft * 4 < (int64_t(1) << 31) &&
+    return a.nz > 1 && a.nz == 2 * a.Z + 1 && a.nstages <= 4 && (int64_t)(a.Z + 16) * a.nfft * 4 < (int64_t(1) << 31) &&
            a.nfft % (TILE_NT * TILE_HP) == 0 && a.nfft / (TILE_NT * TILE_HP) <= 65535 && a.nb <= 65535;
+}
+
+// Where tiles gain: planes of 32 MB and more, whose rows come from L2 or HBM anew for every harmonic.  Whole searches
+// of 128 trials, 8 harmonics, row kernel and tiles: 53 MB planes 8.23 -> 7.82 ms (51 rows) and 8.09 -> 7.47 ms (201
+// rows), 106 MB 14.50 -> 13.36 ms, 211 MB 29.3 -> 26.5 ms; 26 MB 4.54 and 4.52 ms, 13 MB 2.82 and 2.93 ms.  Rows of
+// the last tile past the edge are summed in vain: at most 0.3 times the plane's.
+bool tile_gains(const HarmArgs& a) {
+    const int64_t rows = 2 * TILE_RT * (int64_t)((a.Z + TILE_RT) / TILE_RT);
+    return 10 * rows <= 13 * (int64_t)a.nz && (int64_t)a.nz * a.nfft * 4 >= (int64_t(32) << 20);
 }
 
 template <int NSTAGES>
 cudaError_t launch_tile_t(const HarmArgs& a, cudaStream_t s) {
-    constexpr int RT = TileRows<NSTAGES>::value;
-    dim3 grid((unsigned)(2 * ((a.Z + RT) / RT)), (unsigned)(a.nfft / (TILE_NT * TILE_HP)), (unsigned)a.nb);
+    dim3 grid((unsigned)(2 * ((a.Z + TILE_RT) / TILE_RT)), (unsigned)(a.nfft / (TILE_NT * TILE_HP)), (unsigned)a.nb);
     k_harm_tile<NSTAGES><<<grid, TILE_NT, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -433,19 +438,18 @@ cudaError_t launch_tile(const HarmArgs& a, cudaStream_t s) {
         case 2: return launch_tile_t<2>(a, s);
         case 3: return launch_tile_t<3>(a, s);
         case 4: return launch_tile_t<4>(a, s);
-        case 5: return launch_tile_t<5>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
-// 2-D planes: the warps of a block take consecutive plane rows (default; 31.1 -> 28.9 ms on
-// the zmax 200 accel file); PSS_HARM_ROWS=0 keeps one row per block
-bool harm_rows() {
+// 2-D planes: tiles of rows where they gain, else the warps of a block take consecutive plane rows (31.1 -> 28.9 ms on
+// the zmax 200 accel file).  PSS_HARM_ROWS=0: one row per block; 1: tiles wherever they can run.
+int harm_rows() {
     static const int v = [] {
         const char* e = getenv("PSS_HARM_ROWS");
-        return e ? (e[0] == '1' ? 1 : 0) : 1;
+        return e ? (e[0] == '1' ? 1 : 0) : 2;
     }();
-    return v == 1;
+    return v;
 }
 
 template <int R, bool ROWS>
@@ -476,7 +480,7 @@ cudaError_t launch_reg(const HarmArgs& a, cudaStream_t s) {
 cudaError_t launch_harm(const HarmArgs& a, cudaStream_t s) {
     if (a.nfft > (int64_t(1) << 24) || a.nstages > 6) return cudaErrorInvalidValue;
     if ((int64_t)a.nz * a.nfft > (int64_t(1) << 31)) return cudaErrorInvalidValue;  // 32-bit plane offsets
-    if (harm_rows() && tile_usable(a)) return launch_tile(a, s);
+    if (harm_rows() && tile_usable(a) && (harm_rows() == 1 || tile_gains(a))) return launch_tile(a, s);
     // register-blocked kernel: up to 16 harmonics, whole warps of 32 x 16 points
     if (a.run == 8 && a.nstages <= 5 && a.nfft % (REG_NT * 8) == 0 && a.nfft / (REG_NT * 8) <= 65535 &&
         a.nb <= 65535)
