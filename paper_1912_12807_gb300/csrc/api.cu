@@ -1203,6 +1203,7 @@ pss_status enqueue_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
                     pl.twM = ctx->twid_n;
                     pl.nz = P.nz;
                     pl.form = ctx->tune.plane_form;
+                    pl.num_sms = ctx->num_sms;
                     pl.zrow0 = -1;
                     for (int j = 0; j < P.nz; ++j)
                         if (-(double)cfg->zmax + (double)j * pl.dz == 0.0) pl.zrow0 = j;
@@ -1735,6 +1736,7 @@ pss_status multi_enqueue(pss_ctx* ctx, const pss_search_cfg* cfg, const MultiSet
                 pl.twM = ctx->twid_n;
                 pl.nz = M.nz;
                 pl.form = ctx->tune.plane_form;
+                pl.num_sms = ctx->num_sms;
                 pl.zrow0 = -1;
                 for (int j = 0; j < M.nz; ++j)
                     if (-(double)cfg->zmax + (double)j * pl.dz == 0.0) pl.zrow0 = j;

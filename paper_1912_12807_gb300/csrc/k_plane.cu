@@ -437,15 +437,20 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
 // straight to the plane.
 //
 // Bound by the chain load - butterfly - barrier of a row with 16 warps per SM
-// (registers), not by a unit: leaving out the template loads, the
-// twiddles, the arithmetic or the stores saves 5 to 16 % each.  So the first
-// F16PRE template quads of the next row are loaded before the last sub-stage.
-// 301 trials x 201 rows of 2^18 (with the harmonic sums and the rest of the
-// search): 62.3 ms with scalar arithmetic, 61.5 packed, 61.25 with 4 quads
-// loaded ahead (8: 62.8, spills); 8 trials x 201 rows of 2^18 (plane call):
-// 1203 -> 1192 -> 1181 us.
+// (128 registers a thread), not by a unit: leaving out the template loads, the
+// twiddles, the arithmetic or the stores saves 5 to 16 % each.  The loop keeps
+// two pointers and its bins; even so 20 words are spilled in the set-up and 10
+// of them read back per row (ptxas: 80 bytes of spill stores, 40 of loads).
+// Template quads of the next row loaded ahead, and the z = 0 row handled in the
+// loop, cost more spills than they hide: 112 bytes and 56 with four quads.
+// 64 trials x 201 rows of 2^18 (plane alone): 7.87 ms with scalar arithmetic,
+// 7.58 packed with four quads ahead, 7.31 here; 64 x 101 rows of 2^16 1.034,
+// 1.030 and 0.987 ms; 4 x 101 rows of 2^16, one CTA per segment, 0.260, 0.276
+// and 0.278 ms (the rows of so few are split: fft16_rows).
 constexpr int F16NT = 128;
-constexpr int F16PRE = 4;           // template quads of the next row loaded ahead
+constexpr int F16CTAS = 4;          // CTAs per SM
+constexpr int F16MAXSPLIT = 8;      // row ranges of a segment at most
+constexpr double F16SETUP = 8.0;    // a CTA's set-up (twiddle tables, the segment's spectrum) in rows
 constexpr int T16A = 0;             // RR 16, NS 16: 16 x 16
 constexpr int T16B = T16A + 256;    // RR 8, NS 256: 8 x 256
 constexpr int T16N = T16B + 2048;
@@ -549,7 +554,8 @@ __device__ __forceinline__ void last8(const float4* Y, const float2* tl, int bb,
     dft8(x);
 }
 
-__global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant__ PlaneArgs a) {
+// Rows rows_per blockIdx.z .. + rows_per - 1 of segment blockIdx.x of trial blockIdx.y.
+__global__ void __launch_bounds__(F16NT, F16CTAS) k_plane_fft16(const __grid_constant__ PlaneArgs a, int rows_per) {
     constexpr int L = PLANE_FFT_L;
     constexpr int NE = L / F16NT;  // 16 bins per thread
     extern __shared__ float4 f16sm[];
@@ -596,20 +602,18 @@ __global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant_
         }
     }
     __syncthreads();
-    const int nz = a.nz;
-    float2* P = reinterpret_cast<float2*>(a.plane + (int64_t)b * a.plane_stride);
-    float4 tp[F16PRE];
-#pragma unroll
-    for (int e = 0; e < F16PRE; ++e) tp[e] = __ldg(reinterpret_cast<const float4*>(a.ftaps) + threadIdx.x + e * F16NT);
-    for (int j = 0; j < nz; ++j) {
-        const bool zrow0 = (j == a.zrow0);
-        const float4* T = reinterpret_cast<const float4*>(a.ftaps + (int64_t)j * 2 * L) + threadIdx.x;
+    const int j_lo = blockIdx.z * rows_per, j_hi = min(a.nz, j_lo + rows_per);
+    const float4* T = reinterpret_cast<const float4*>(a.ftaps + (int64_t)j_lo * 2 * L) + threadIdx.x;
+    float2* row = reinterpret_cast<float2*>(a.plane + (int64_t)b * a.plane_stride) + (int64_t)j_lo * M + k0;
+    const int left = (int)min((int64_t)V, M - k0);
+#pragma unroll 1
+    for (int j = j_lo; j < j_hi; ++j) {
         {
             cc x[NE];
 #pragma unroll
             for (int e = 0; e < NE; ++e) {
                 // conj(X T) of both parities
-                const float4 t = e < F16PRE ? tp[e < F16PRE ? e : 0] : __ldg(T + e * F16NT);
+                const float4 t = __ldg(T + e * F16NT);
                 const float2 tr = make_float2(t.x, t.y), ti = make_float2(t.z, t.w);
                 const float2 xr = make_float2(X[e].x, X[e].x), nxr = make_float2(-X[e].x, -X[e].x);
                 const float2 nxi = make_float2(-X[e].y, -X[e].y);
@@ -621,12 +625,6 @@ __global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant_
         }
         __syncthreads();
         mid16(Y, twt + T16A);
-        if (j + 1 < nz) {
-#pragma unroll
-            for (int e = 0; e < F16PRE; ++e) tp[e] = __ldg(T + 2048 + e * F16NT);
-        }
-        float2* row = P + (int64_t)j * M + k0;
-        const int left = (int)min((int64_t)V, M - k0);
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             const int bb = threadIdx.x + p * F16NT;
@@ -635,15 +633,39 @@ __global__ void __launch_bounds__(F16NT, 4) k_plane_fft16(const __grid_constant_
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int u = bb + q * 256;
-                if (u < left) {
-                    float2 pw = fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re));
-                    if (zrow0) pw.x = pow2(Ap[k0 + u]);  // integer half-bins of the z = 0 row: the raw powers, exactly
-                    row[u] = pw;
-                }
+                if (u < left) row[u] = fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re));
             }
         }
+        T += L;
+        row += M;
         __syncthreads();  // the next row's first sub-stage overwrites Y
     }
+    // integer half-bins of the z = 0 row: the raw powers, exactly (each thread over what it wrote itself)
+    if (a.zrow0 >= j_lo && a.zrow0 < j_hi) {
+        row -= (int64_t)(j_hi - a.zrow0) * M;
+        for (int u = threadIdx.x; u < left; u += F16NT) row[u].x = pow2(Ap[k0 + u]);
+    }
+}
+
+// Rows per CTA: the segments' rows are split over up to 8 CTAs where that shortens the run by 5 % or more, counted in
+// waves of F16CTAS CTAs per SM that each take their rows and the set-up (8 rows: from the times of planes of one
+// trial, unsplit and in 8 ranges).  Planes of a few trials are below one wave (one trial of 2^18: 73 of 608 CTAs),
+// and a batch's last wave may be nearly empty.  Measured, scalar arithmetic of one CTA per segment / packed, unsplit /
+// split: one trial x 201 rows of 2^18 0.512 / 0.543 / 0.145 ms, of 2^14 0.389 / 0.413 / 0.067 ms; 4 trials of 2^18
+// 0.602 / 0.582 / 0.508 ms; 29 trials x 101 rows of 2^18 (3.3 waves) 1.825 / 1.720 / 1.657 ms.
+int fft16_rows(int64_t ctas, int nz, int num_sms) {
+    const int64_t slots = (int64_t)(num_sms > 0 ? num_sms : 152) * F16CTAS;
+    int rows_per = nz;
+    double best = 1e300;
+    for (int split = 1; split <= F16MAXSPLIT && split <= nz; ++split) {
+        const int rows = (nz + split - 1) / split, ranges = (nz + rows - 1) / rows;
+        const double t = (double)((ctas * ranges + slots - 1) / slots) * (rows + F16SETUP);
+        if (t < 0.95 * best) {
+            best = t;
+            rows_per = rows;
+        }
+    }
+    return rows_per;
 }
 
 }  // namespace
@@ -684,8 +706,10 @@ cudaError_t launch_plane(const PlaneArgs& a, cudaStream_t s) {
         const size_t shm = (size_t)PLANE_FFT_L * sizeof(float4) + T16N * sizeof(float2);
         cudaError_t e = allow_smem((const void*)k_plane_fft16, shm);
         if (e != cudaSuccess) return e;
-        dim3 grid((unsigned)((M + a.fV - 1) / a.fV), (unsigned)a.nb);
-        k_plane_fft16<<<grid, F16NT, shm, s>>>(a);
+        const int64_t segs = (M + a.fV - 1) / a.fV;
+        const int rows_per = fft16_rows(segs * a.nb, a.nz, a.num_sms);
+        dim3 grid((unsigned)segs, (unsigned)a.nb, (unsigned)((a.nz + rows_per - 1) / rows_per));
+        k_plane_fft16<<<grid, F16NT, shm, s>>>(a, rows_per);
         return cudaGetLastError();
     }
     if (a.ftaps) {

@@ -652,6 +652,7 @@ struct PlaneArgs {
     int32_t fL, fV, fM0;     // segment length, valid outputs per segment, lead
     int32_t nz, zrow0;       // rows, and the row with z = 0 exactly (-1: none)
     int32_t form;            // overlap-save FFT: 0 radix 8-8-8-4 (256 threads), 1 radix 16-16-8 (128 threads)
+    int32_t num_sms;         // SMs of the device (0: unknown)
     const float2* tw;        // exp(-2 pi i t / twM)
     int64_t twM;
 };
