@@ -416,13 +416,20 @@ bool tile_usable(const HarmArgs& a) {
            a.nfft % (TILE_NT * TILE_HP) == 0 && a.nfft / (TILE_NT * TILE_HP) <= 65535 && a.nb <= 65535;
 }
 
-// Where tiles gain: planes of 32 MB and more, whose rows come from L2 or HBM anew for every harmonic.  Whole searches
-// of 128 trials, 8 harmonics, row kernel and tiles: 53 MB planes 8.23 -> 7.82 ms (51 rows) and 8.09 -> 7.47 ms (201
-// rows), 106 MB 14.50 -> 13.36 ms, 211 MB 29.3 -> 26.5 ms; 26 MB 4.54 and 4.52 ms, 13 MB 2.82 and 2.93 ms.  Rows of
-// the last tile past the edge are summed in vain: at most 0.3 times the plane's.
+// Where tiles gain: many trials of large planes, whose rows come from L2 or HBM anew for every harmonic.  A launch of
+// tiles starts and drains about 0.03 ms slower than one of rows (fewer, longer warps), and a trial of it is shorter by
+// a time that grows faster than the plane (more of it is out of L2): break-even is at 30 to 60 trials of 50 MiB, 5 to
+// 9 of 100 MiB and 1 to 3 of 200 MiB, and below 40 MiB it is not reached with the trials that a batch can hold.
+// Kernel times, rows and tiles, 8 harmonics: 51 rows of 2^18 (51 MiB) 16 trials 0.348 and 0.373 ms, 128 trials 2.65
+// and 2.49; 201 rows of 2^16 (50 MiB) 32 trials 0.741 and 0.821, 128 trials 2.73 and 2.49; 101 rows of 2^17 (50 MiB) 32
+// trials 0.684 and 0.718, 64 trials 1.348 and 1.290; 101 rows of 2^18 (101 MiB) 4 trials 0.180 and 0.188, 16 trials
+// 0.678 and 0.604; 101 rows of 2^19 (202 MiB) 2 trials 0.201 and 0.221, 4 trials 0.387 and 0.375; 201 rows of 2^18
+// (201 MiB) 4 trials 0.381 and 0.328; 201 rows of 2^19 (402 MiB) 1 trial 0.229 and 0.195; 35 rows of 2^18 (35 MiB) 128
+// trials 1.83 and 1.87.  Rows of the last tile past the edge are summed in vain: at most 0.3 times the plane's.
 bool tile_gains(const HarmArgs& a) {
     const int64_t rows = 2 * TILE_RT * (int64_t)((a.Z + TILE_RT) / TILE_RT);
-    return 10 * rows <= 13 * (int64_t)a.nz && (int64_t)a.nz * a.nfft * 4 >= (int64_t(32) << 20);
+    const double mib = (double)a.nz * (double)a.nfft * 4.0 / 1048576.0;
+    return 10 * rows <= 13 * (int64_t)a.nz && mib >= 32.0 && a.nb * (mib / 50.0) * (mib / 50.0) >= 64.0;
 }
 
 template <int NSTAGES>
