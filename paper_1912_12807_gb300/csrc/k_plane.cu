@@ -439,14 +439,13 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
 // Bound by the chain load - butterfly - barrier of a row with 16 warps per SM
 // (128 registers a thread), not by a unit: leaving out the template loads, the
 // twiddles, the arithmetic or the stores saves 5 to 16 % each.  The loop keeps
-// two pointers and its bins; even so 20 words are spilled in the set-up and 10
-// of them read back per row (ptxas: 80 bytes of spill stores, 40 of loads).
-// Template quads of the next row loaded ahead, and the z = 0 row handled in the
-// loop, cost more spills than they hide: 112 bytes and 56 with four quads.
-// 64 trials x 201 rows of 2^18 (plane alone): 7.87 ms with scalar arithmetic,
-// 7.58 packed with four quads ahead, 7.31 here; 64 x 101 rows of 2^16 1.034,
-// 1.030 and 0.987 ms; 4 x 101 rows of 2^16, one CTA per segment, 0.260, 0.276
-// and 0.278 ms (the rows of so few are split: fft16_rows).
+// two pointers and its bins; even so 21 words are spilled in the set-up and 12
+// read back (ptxas: 84 bytes of spill stores, 48 of loads).  Template quads of
+// the next row loaded ahead, or the z = 0 row tested where its powers are
+// written, cost more spills than they hide (112 and 56 bytes).
+// Planes alone, scalar arithmetic / packed with four quads loaded ahead / here:
+// 64 trials x 201 rows of 2^18 7.87 / 7.58 / 7.08 ms, of 2^16 2.10 / 2.00 /
+// 1.92 ms; 8 trials x 21 rows of 2^18 0.127 / 0.125 / 0.119 ms.
 constexpr int F16NT = 128;
 constexpr int F16CTAS = 4;          // CTAs per SM
 constexpr int F16MAXSPLIT = 8;      // row ranges of a segment at most
@@ -625,34 +624,45 @@ __global__ void __launch_bounds__(F16NT, F16CTAS) k_plane_fft16(const __grid_con
         }
         __syncthreads();
         mid16(Y, twt + T16A);
+        if (j != a.zrow0) {
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const int bb = threadIdx.x + p * F16NT;
-            cc x[8];
-            last8(Y, twt + T16B, bb, x);
+            for (int p = 0; p < 2; ++p) {
+                const int bb = threadIdx.x + p * F16NT;
+                cc x[8];
+                last8(Y, twt + T16B, bb, x);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int u = bb + q * 256;
-                if (u < left) row[u] = fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re));
+                for (int q = 0; q < 8; ++q) {
+                    const int u = bb + q * 256;
+                    if (u < left) row[u] = fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re));
+                }
+            }
+        } else {
+            // integer half-bins of the z = 0 row: the raw powers, exactly
+            const float2* c = a.spec + (int64_t)b * a.spec_stride + k0;
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+                const int bb = threadIdx.x + p * F16NT;
+                cc x[8];
+                last8(Y, twt + T16B, bb, x);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int u = bb + q * 256;
+                    if (u < left) row[u] = make_float2(pow2(c[u]), fma2(x[q].im, x[q].im, mul2(x[q].re, x[q].re)).y);
+                }
             }
         }
         T += L;
         row += M;
         __syncthreads();  // the next row's first sub-stage overwrites Y
     }
-    // integer half-bins of the z = 0 row: the raw powers, exactly (each thread over what it wrote itself)
-    if (a.zrow0 >= j_lo && a.zrow0 < j_hi) {
-        row -= (int64_t)(j_hi - a.zrow0) * M;
-        for (int u = threadIdx.x; u < left; u += F16NT) row[u].x = pow2(Ap[k0 + u]);
-    }
 }
 
 // Rows per CTA: the segments' rows are split over up to 8 CTAs where that shortens the run by 5 % or more, counted in
 // waves of F16CTAS CTAs per SM that each take their rows and the set-up (8 rows: from the times of planes of one
 // trial, unsplit and in 8 ranges).  Planes of a few trials are below one wave (one trial of 2^18: 73 of 608 CTAs),
-// and a batch's last wave may be nearly empty.  Measured, scalar arithmetic of one CTA per segment / packed, unsplit /
-// split: one trial x 201 rows of 2^18 0.512 / 0.543 / 0.145 ms, of 2^14 0.389 / 0.413 / 0.067 ms; 4 trials of 2^18
-// 0.602 / 0.582 / 0.508 ms; 29 trials x 101 rows of 2^18 (3.3 waves) 1.825 / 1.720 / 1.657 ms.
+// and a batch's last wave may be nearly empty.  Measured, 201 rows, scalar arithmetic and one CTA per segment / packed
+// and one CTA per segment / here: 2 trials of 2^16 0.496 / 0.526 / 0.104 ms, 2 trials of 2^18 0.534 / 0.561 / 0.254
+// ms, 4 trials 0.598 / 0.627 / 0.496 ms, 29 trials (3.5 waves) 3.61 / 3.51 / 3.24 ms.
 int fft16_rows(int64_t ctas, int nz, int num_sms) {
     const int64_t slots = (int64_t)(num_sms > 0 ? num_sms : 152) * F16CTAS;
     int rows_per = nz;
