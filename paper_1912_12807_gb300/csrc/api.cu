@@ -211,13 +211,26 @@ pss_status ensure_bx(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_t dm_
     return PSS_OK;
 }
 
+pss_status ensure_errflag(pss_ctx* ctx, cudaStream_t s) {
+    if (ctx->errflag.p) return PSS_OK;
+    PSS_TRY(ctx->errflag.ensure(sizeof(int)));
+    PSS_CUDA(cudaMemsetAsync(ctx->errflag.p, 0, sizeof(int), s));
+    return PSS_OK;
+}
+
+// The unpacked file's buffers: channel-major bytes, rows of bits.
+pss_status ensure_unpacked(pss_ctx* ctx, const pss_fil_desc* fil, int32_t ck, int64_t pitch, bool bytes, bool bits) {
+    if (bytes) PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
+    if (bits) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
+    return PSS_OK;
+}
+
 // Host-side set-up for a file: the kept channels, their delays for
 // [dm_begin, dm_end) (or the two-stage tables, `T`) uploaded to
 // ctx->delays_dev, and the channel-major buffer.  Synchronises `s` (the
 // delay upload reads a host vector).
 pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin,
-                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr,
-                       bool bx = true) {
+                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr) {
     // a call that fails part-way may have replaced the tables or given up a buffer: set-ups kept for them end
     struct Done {
         pss_ctx* ctx;
@@ -255,11 +268,8 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
     }
     PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
     if (fil->nbits == 1 && plan->nsub == 0 && ck <= 255) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
-    if (bx) PSS_TRY(ensure_bx(ctx, plan, ck, dm_begin, dm_end));
-    if (!ctx->errflag.p) {
-        PSS_TRY(ctx->errflag.ensure(sizeof(int)));
-        PSS_CUDA(cudaMemsetAsync(ctx->errflag.p, 0, sizeof(int), s));
-    }
+    PSS_TRY(ensure_bx(ctx, plan, ck, dm_begin, dm_end));
+    PSS_TRY(ensure_errflag(ctx, s));
     if (!same) {
         PSS_CUDA(cudaStreamSynchronize(s));  // `host` is about to go out of scope
         ctx->delays_host.swap(host);
@@ -286,14 +296,14 @@ pss_status upload_input(pss_ctx* ctx, const pss_fil_desc* fil, const void* data,
 // Unpack/transpose the file into ctx->xcm, or, as rows of bits, into
 // ctx->xbits (kernel launches only).
 pss_status enqueue_prep(pss_ctx* ctx, const pss_fil_desc* fil, const uint8_t* src, int32_t ck, int64_t pitch,
-                        cudaStream_t s, bool bytes = true, bool bits = false) {
+                        cudaStream_t s, bool bytes = true, bool bits = false, const int32_t* keep = nullptr) {
     PrepArgs pa;
     pa.src = src;
     pa.nchan = fil->nchan;
     pa.nbits = fil->nbits;
     pa.layout = fil->layout;
     pa.nsamp = fil->nsamp;
-    pa.keep = (const int32_t*)ctx->delays_dev.p;
+    pa.keep = keep ? keep : (const int32_t*)ctx->delays_dev.p;
     pa.ck = ck;
     pa.xcm = (uint8_t*)ctx->xcm.p;
     pa.pitch = pitch;
@@ -433,13 +443,14 @@ pss_status dd_upload(pss_ctx* ctx, int which, const std::vector<uint8_t>& host, 
 // Dedisperse trials [b0, b0 + nb) of one stage into rows of out_stride
 // (float out_f with per-trial sums, or int32 out_i): the exact kernel, or,
 // for a two-stage plan, stage 1 into `subu` and stage 2 from it.  `spread`
-// is the exact kernel's delay spread; `SB` the two-stage launch sizes.
+// is the exact kernel's delay spread; `SB` the two-stage launch sizes; `tab`
+// the device tables (ctx->delays_dev unless given; its first trial is dm_begin).
 pss_status enqueue_dedisp(pss_ctx* ctx, const pss_plan* plan, int32_t ck, int64_t pitch, const SubTab& T,
                           const StageInfo& st, int64_t dm_begin, int64_t b0, int32_t nb, int32_t spread,
                           const SubBatch& SB, const DdBatch& dd, void* subu, float* out_f,
                           int32_t* out_i, int64_t out_stride, unsigned long long* sums, cudaStream_t s,
-                          unsigned long long* squares = nullptr) {
-    const int32_t* base = (const int32_t*)ctx->delays_dev.p;
+                          unsigned long long* squares = nullptr, const int32_t* tab = nullptr) {
+    const int32_t* base = tab ? tab : (const int32_t*)ctx->delays_dev.p;
     if (!T.on && dd.kind == DD_BITS) {
         B1Args ba{};
         ba.xb = (const uint8_t*)ctx->xbits.p;
@@ -882,10 +893,8 @@ std::string path_key(const pss_plan* plan, const pss_fil_desc* fil, const pss_se
 // Host set-up of a plain dedispersion (pss_dedisperse, pss_single_pulse) of
 // [dm_begin, dm_end): input tables, DM batches, shared-sum tables and the
 // stage-1 buffer, kept like PathCache while the request is the same and the
-// device tables are still the ones uploaded for it.  pss_fold keeps the input
-// tables of the whole plan (its trials change from call to call), which are
-// those of a search of the whole plan.
-enum DdUse { DD_DEDISPERSE, DD_SINGLE_PULSE, DD_FOLD };
+// device tables are still the ones uploaded for it.
+enum DdUse { DD_DEDISPERSE, DD_SINGLE_PULSE };
 
 struct DdSetup {
     std::string key;
@@ -896,8 +905,6 @@ struct DdSetup {
     std::vector<BatchDesc> batches;  // out_off: samples of the trials before, packed
     size_t need_subu = 0;
     bool need_bytes = false, need_bits = false;
-    std::vector<int32_t> keep;       // pss_fold: the kept channels
-    DdBatch fold;                    // pss_fold: how its runs of trials are dedispersed
 };
 
 pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin, int64_t dm_end,
@@ -905,45 +912,22 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     const pss_search_cfg none{};
     std::string key = path_key(plan, fil, &none, dm_begin, dm_end, MODE_SPECTRUM, (int64_t)use, 0, ctx->tune);
     key_put(&key, ctx->tune.bx_min);
-    std::shared_ptr<void>& slot = use == DD_FOLD ? ctx->fold_cache : ctx->dd_cache;
-    auto kept = std::static_pointer_cast<DdSetup>(slot);
+    auto kept = std::static_pointer_cast<DdSetup>(ctx->dd_cache);
     if (kept && kept->key == key && dm_end > dm_begin) {
         if (kept->gen != ctx->delays_gen) {  // another request's delays are on the device
             SubTab T;
-            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &kept->ck, &kept->pitch, &T, use != DD_FOLD));
+            PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &kept->ck, &kept->pitch, &T));
             kept->gen = ctx->delays_gen;
         }
+        // (another call may have given a buffer up)
+        PSS_TRY(ensure_unpacked(ctx, fil, kept->ck, kept->pitch, kept->need_bytes, kept->need_bits));
         if (kept->need_subu) PSS_TRY(ctx->subu.ensure(kept->need_subu));
         *out = kept;
         return PSS_OK;
     }
     auto D = std::make_shared<DdSetup>();
-    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T, use != DD_FOLD));
+    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T));
     D->need_bytes = D->T.on;
-    if (use == DD_FOLD) {
-        // bit-sliced where any 16 consecutive trials' delays fit (delays are monotonic in DM)
-        D->keep = kept_channels(fil);
-        int32_t spread = 0;
-        for (const auto& st : plan->stages)
-            for (int64_t i = st.first; i + 1 < st.first + st.n_dm; ++i) {
-                const int64_t e = std::min<int64_t>(i + 15, st.first + st.n_dm - 1);
-                for (int32_t c : D->keep)
-                    spread = std::max(spread, std::abs(plan->delays[(size_t)e * plan->nchan + c] - plan->delays[(size_t)i * plan->nchan + c]));
-            }
-        int KW, rowb;
-        size_t shm;
-        if (fil->nbits == 1 && !D->T.on && b1_sizes(spread, D->ck, 16, &KW, &rowb, &shm)) {
-            D->fold.kind = DD_BITS;
-            D->fold.group = 16;
-            D->fold.spread = spread;
-        }
-        (D->fold.kind == DD_BITS ? D->need_bits : D->need_bytes) = true;
-        D->key.swap(key);
-        D->gen = ctx->delays_gen;
-        slot = D;
-        *out = D;
-        return PSS_OK;
-    }
     const std::vector<int32_t> hd = D->T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
     std::vector<uint8_t> dd_host;
     int64_t off = 0;
@@ -981,7 +965,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
     PSS_TRY(dd_upload(ctx, 1, dd_host, s));
     D->key.swap(key);
     D->gen = ctx->delays_gen;
-    slot = D;
+    ctx->dd_cache = D;
     *out = D;
     return PSS_OK;
 }
@@ -998,6 +982,8 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
             PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &pc->P.ck, &pc->P.pitch, &T));
             pc->gen = ctx->delays_gen;
         }
+        // (another call may have given a buffer up)
+        PSS_TRY(ensure_unpacked(ctx, fil, pc->P.ck, pc->P.pitch, pc->P.need_bytes, pc->P.need_bits));
         *P = pc->P;
     } else {
         PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &P->ck, &P->pitch, &P->sub));
@@ -1977,7 +1963,7 @@ void pss_ctx_destroy(pss_ctx* c) {
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     DevBuf* bufs[] = {&c->fil_dev, &c->xcm, &c->xbits, &c->delays_dev, &c->ddtab[0], &c->ddtab[1], &c->subu, &c->sp_series, &c->sp_mom, &c->sp_ev,
-                      &c->fold_buf, &c->bx, &c->mf_fil, &c->mf_xcm, &c->mf_work, &c->series, &c->sums, &c->fftA, &c->fftB,
+                      &c->fold_buf, &c->fold_tab, &c->bx, &c->mf_fil, &c->mf_xcm, &c->mf_work, &c->series, &c->sums, &c->fftA, &c->fftB,
                       &c->spec, &c->plane, &c->cands, &c->counter, &c->taps, &c->ftaps, &c->tapinfo, &c->errflag,
                       &c->twid, &c->chan_spec, &c->refine_gains, &c->refine_dtau, &c->refine_pts, &c->refine_out};
     for (DevBuf* b : bufs) b->release();
@@ -2252,29 +2238,20 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
     PSS_TRY(check_common(ctx, plan, fil, data, lo_dm, hi_dm + 1));
     PSS_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t s = pick_stream(ctx, stream);
-    std::shared_ptr<DdSetup> D;
-    PSS_TRY(setup_dedisp(ctx, plan, fil, 0, plan->ndm(), DD_FOLD, s, &D));
-    PSS_TRY(ensure_bx(ctx, plan, D->ck, lo_dm, hi_dm + 1));  // of the rows folded from only
-    const int32_t ck = D->ck;
-    const uint8_t* src = nullptr;
-    PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
-    PSS_TRY(enqueue_prep(ctx, fil, src, ck, D->pitch, s, D->need_bytes, D->need_bits));
-    // requests by trial; chunks of at most 256 series rows
+    // requests by trial, in chunks of at most MAXROWS series rows: runs of trials of one stage (gaps of at most 15
+    // trials dedispersed as well)
     std::vector<int64_t> order(n);
     for (int64_t i = 0; i < n; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return reqs[a].dm_idx < reqs[b].dm_idx; });
-    int64_t nv_max = 0;
-    for (const auto& st : plan->stages) nv_max = std::max<int64_t>(nv_max, st.nv);
     constexpr int64_t MAXROWS = 256;
-    PSS_TRY(ctx->sp_series.ensure((size_t)MAXROWS * nv_max * sizeof(int32_t)));
-    PSS_TRY(ctx->sp_mom.ensure((size_t)2 * MAXROWS * sizeof(unsigned long long)));
-    size_t q0 = 0;
-    while (q0 < order.size()) {
-        // runs of trials (same stage, gaps of at most 15 trials dedispersed as well) up to MAXROWS rows
-        struct Run { int64_t a, b; int32_t row0; };
-        std::vector<Run> runs;
+    struct Run { int64_t a, b; int32_t row0; int64_t tab0; DdBatch dd; };  // tab0: first row in the delay table
+    struct Chunk { size_t q0, q1; std::vector<Run> runs; };
+    std::vector<Chunk> chunks;
+    int64_t nrows = 0;  // of the delay table
+    for (size_t q = 0; q < order.size();) {
+        Chunk ch{q, q, {}};
+        std::vector<Run>& runs = ch.runs;
         int32_t rows = 0;
-        size_t q = q0;
         while (q < order.size()) {
             const int64_t d = reqs[order[q]].dm_idx;
             if (!runs.empty() && d < runs.back().b) { ++q; continue; }
@@ -2283,13 +2260,77 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
                 rows += (int32_t)(d + 1 - runs.back().b);
                 runs.back().b = d + 1;
             } else if (rows + 1 <= MAXROWS) {
-                runs.push_back({d, d + 1, rows});
+                runs.push_back({d, d + 1, rows, 0, DdBatch()});
                 rows += 1;
             } else {
                 break;
             }
             ++q;
         }
+        for (Run& r : runs) r.tab0 = nrows + r.row0;
+        nrows += rows;
+        ch.q1 = q;
+        chunks.push_back(std::move(ch));
+    }
+    int32_t ck = 0;
+    int64_t pitch = 0;
+    SubTab T;
+    bool bytes = true;
+    const int32_t* tab = nullptr;  // exact plans: the kept channels and the delays of the runs' trials
+    if (plan->nsub > 0) {
+        PSS_TRY(setup_input(ctx, plan, fil, lo_dm, hi_dm + 1, s, &ck, &pitch, &T));
+    } else {
+        // a table of the folded trials alone, beside the one that searches and dedispersions keep
+        const std::vector<int32_t> keep = kept_channels(fil);
+        ck = (int32_t)keep.size();
+        if (ck == 0) return fail(PSS_EINVAL, "channel mask removes every channel");
+        pitch = xcm_pitch(*plan, fil);
+        std::vector<int32_t> host(keep);
+        host.reserve((size_t)(1 + nrows) * ck);
+        for (const Chunk& ch : chunks)
+            for (const Run& r : ch.runs) {
+                const std::vector<int32_t> hd = compact_delays(plan, keep, r.a, r.b);
+                host.insert(host.end(), hd.begin(), hd.end());
+            }
+        // bit-sliced where the delays of every run fit
+        bytes = fil->nbits != 1;
+        for (Chunk& ch : chunks)
+            for (Run& r : ch.runs) {
+                const int32_t* rows = host.data() + ck + r.tab0 * ck;
+                const int32_t nb = (int32_t)(r.b - r.a);
+                r.dd.group = fil->nbits == 1 ? 16 : 0;
+                r.dd.spread = fil->nbits == 1 ? delay_spread(rows, nb, ck, 16) : delay_spread(rows, nb, ck);
+                int KW, rowb;
+                size_t shm;
+                if (!bytes && !b1_sizes(r.dd.spread, ck, 16, &KW, &rowb, &shm)) bytes = true;
+            }
+        for (Chunk& ch : chunks)
+            for (Run& r : ch.runs) {
+                r.dd.kind = bytes ? DD_DIRECT : DD_BITS;
+                if (bytes && fil->nbits == 1) r.dd.spread = delay_spread(host.data() + ck + r.tab0 * ck, r.b - r.a, ck);
+            }
+        const void* before = ctx->fold_tab.p;
+        PSS_TRY(ctx->fold_tab.ensure(host.size() * sizeof(int32_t)));
+        if (ctx->fold_tab.p != before || ctx->fold_host != host) {
+            ctx->fold_host.clear();
+            PSS_CUDA(cudaMemcpyAsync(ctx->fold_tab.p, host.data(), host.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+            PSS_CUDA(cudaStreamSynchronize(s));  // `host` may go
+            ctx->fold_host.swap(host);
+        }
+        tab = (const int32_t*)ctx->fold_tab.p;
+        PSS_TRY(ensure_unpacked(ctx, fil, ck, pitch, bytes, !bytes));
+        PSS_TRY(ensure_bx(ctx, plan, ck, lo_dm, hi_dm + 1));
+        PSS_TRY(ensure_errflag(ctx, s));
+    }
+    const uint8_t* src = nullptr;
+    PSS_TRY(upload_input(ctx, fil, data, data_on_device, s, &src));
+    PSS_TRY(enqueue_prep(ctx, fil, src, ck, pitch, s, bytes, !bytes, tab));
+    int64_t nv_max = 0;
+    for (const auto& st : plan->stages) nv_max = std::max<int64_t>(nv_max, st.nv);
+    PSS_TRY(ctx->sp_series.ensure((size_t)MAXROWS * nv_max * sizeof(int32_t)));
+    PSS_TRY(ctx->sp_mom.ensure((size_t)2 * MAXROWS * sizeof(unsigned long long)));
+    for (const Chunk& ch : chunks) {
+        const std::vector<Run>& runs = ch.runs;
         int32_t* ser = (int32_t*)ctx->sp_series.p;
         unsigned long long* m1 = (unsigned long long*)ctx->sp_mom.p;
         unsigned long long* m2 = m1 + MAXROWS;
@@ -2297,18 +2338,16 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
         for (const Run& r : runs) {
             const StageInfo& st = plan->stages[plan->stage_of[r.a]];
             const int32_t nb = (int32_t)(r.b - r.a);
-            int32_t spread = 0;
             SubBatch SB;
-            if (D->T.on) {
-                SB = sub_batch(plan, D->T, ck, 0, r.a, nb, st.nv, st.ds);
+            if (T.on) {
+                SB = sub_batch(plan, T, ck, lo_dm, r.a, nb, st.nv, st.ds);
                 PSS_TRY(ctx->subu.ensure((size_t)plan->nsub * SB.ngb * SB.stride1 * 4 + subsum_slack_bytes(SB.spread2)));
-            } else if (D->fold.kind == DD_DIRECT) {
-                spread = delay_spread(compact_delays(plan, D->keep, r.a, r.b).data(), nb, ck);
             }
             int32_t* out = ser + (int64_t)r.row0 * nv_max;
-            const bool mom = D->fold.kind == DD_BITS;  // the bit-sliced kernel forms the moments with the series
-            PSS_TRY(enqueue_dedisp(ctx, plan, ck, D->pitch, D->T, st, 0, r.a, nb, spread, SB, D->fold, ctx->subu.p, nullptr,
-                                   out, nv_max, mom ? m1 + r.row0 : nullptr, s, mom ? m2 + r.row0 : nullptr));
+            const bool mom = !bytes;  // the bit-sliced kernel forms the moments with the series
+            PSS_TRY(enqueue_dedisp(ctx, plan, ck, pitch, T, st, T.on ? lo_dm : r.a - r.tab0, r.a, nb, r.dd.spread, SB, r.dd,
+                                   ctx->subu.p, nullptr, out, nv_max, mom ? m1 + r.row0 : nullptr, s,
+                                   mom ? m2 + r.row0 : nullptr, tab));
             if (!mom) PSS_CUDA(launch_sp_moments(out, nv_max, st.nv, nb, m1 + r.row0, m2 + r.row0, s));
         }
         std::vector<unsigned long long> mom((size_t)2 * MAXROWS);
@@ -2318,7 +2357,7 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
         // items of this chunk's requests
         std::vector<FoldItem> items;
         std::vector<int64_t> which;
-        for (size_t k = q0; k < q; ++k) {
+        for (size_t k = ch.q0; k < ch.q1; ++k) {
             const pss_fold_req& rq = reqs[order[k]];
             int32_t row = -1;
             for (const Run& r : runs)
@@ -2377,7 +2416,6 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
             memcpy(profiles + w * nbin, hp + (i * nfreq + best) * nbin, (size_t)nbin * 8);
             memcpy(counts + w * nbin, hc + (i * nfreq + best) * nbin, (size_t)nbin * 8);
         }
-        q0 = q;
     }
     return PSS_OK;
 }

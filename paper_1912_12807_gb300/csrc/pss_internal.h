@@ -194,7 +194,8 @@ struct Ctx {
     uint64_t delays_gen = 0;           // bumped whenever delays_dev is rewritten
     std::shared_ptr<void> path_cache;  // last search set-up (api.cu), valid while delays_gen matches
     std::shared_ptr<void> dd_cache;    // last set-up of pss_dedisperse / pss_single_pulse, likewise
-    std::shared_ptr<void> fold_cache;  // last set-up of pss_fold, likewise
+    DevBuf fold_tab;                   // int32: kept channels and delays of the trials folded last (exact plans)
+    std::vector<int32_t> fold_host;    // what fold_tab holds, empty if unknown
     DevBuf xbits;        // rows of bits of a 1-bit file (bit-sliced dedispersion)
     DevBuf ddtab[2];     // tables of the shared-sum dedispersion: the search path's batches, the plain calls'
     DevBuf series;       // float [B][nfft]
