@@ -138,6 +138,8 @@ std::vector<int32_t> kept_channels(const pss_fil_desc* fil) {
 std::vector<int32_t> compact_delays(const pss_plan* plan, const std::vector<int32_t>& keep, int64_t dm_begin,
                                     int64_t dm_end) {
     const size_t ck = keep.size();
+    if ((int64_t)ck == plan->nchan)
+        return std::vector<int32_t>(plan->delays.begin() + dm_begin * (int64_t)ck, plan->delays.begin() + dm_end * (int64_t)ck);
     std::vector<int32_t> hd((size_t)(dm_end - dm_begin) * ck);
     for (int64_t i = 0; i < dm_end - dm_begin; ++i)
         for (size_t r = 0; r < ck; ++r)
@@ -225,12 +227,30 @@ pss_status ensure_unpacked(pss_ctx* ctx, const pss_fil_desc* fil, int32_t ck, in
     return PSS_OK;
 }
 
+// Uploads from host vectors of the context that are still to be waited for
+// (a call that fails in between waits too: the vectors may change after it).
+struct Uploads {
+    cudaStream_t s;
+    bool pending = false;
+    explicit Uploads(cudaStream_t str) : s(str) {}
+    pss_status wait() {
+        if (!pending) return PSS_OK;
+        pending = false;
+        PSS_CUDA(cudaStreamSynchronize(s));
+        return PSS_OK;
+    }
+    ~Uploads() {
+        if (pending) cudaStreamSynchronize(s);
+    }
+};
+
 // Host-side set-up for a file: the kept channels, their delays for
 // [dm_begin, dm_end) (or the two-stage tables, `T`) uploaded to
 // ctx->delays_dev, and the channel-major buffer.  Synchronises `s` (the
-// delay upload reads a host vector).
+// delay upload reads a host vector), or leaves that to `up`.
 pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin,
-                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr) {
+                       int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr,
+                       Uploads* up = nullptr) {
     // a call that fails part-way may have replaced the tables or given up a buffer: set-ups kept for them end
     struct Done {
         pss_ctx* ctx;
@@ -261,20 +281,20 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
     const void* before = ctx->delays_dev.p;
     PSS_TRY(ctx->delays_dev.ensure(host.size() * sizeof(int32_t)));
     const bool same = ctx->delays_dev.p == before && ctx->delays_host == host;
+    Uploads own(s);
+    if (!up) up = &own;
     if (!same) {
-        ctx->delays_host.clear();
-        PSS_CUDA(cudaMemcpyAsync(ctx->delays_dev.p, host.data(), host.size() * sizeof(int32_t),
+        ctx->delays_host.swap(host);
+        up->pending = true;
+        PSS_CUDA(cudaMemcpyAsync(ctx->delays_dev.p, ctx->delays_host.data(), ctx->delays_host.size() * sizeof(int32_t),
                                  cudaMemcpyHostToDevice, s));
+        ctx->delays_gen++;
     }
     PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
     if (fil->nbits == 1 && plan->nsub == 0 && ck <= 255) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
     PSS_TRY(ensure_bx(ctx, plan, ck, dm_begin, dm_end));
     PSS_TRY(ensure_errflag(ctx, s));
-    if (!same) {
-        PSS_CUDA(cudaStreamSynchronize(s));  // `host` is about to go out of scope
-        ctx->delays_host.swap(host);
-        ctx->delays_gen++;
-    }
+    PSS_TRY(own.wait());
     done.ok = true;
     *ck_out = ck;
     *pitch_out = pitch;
@@ -320,16 +340,19 @@ pss_status enqueue_prep(pss_ctx* ctx, const pss_fil_desc* fil, const uint8_t* sr
 // channels of (dmax - dmin)
 int32_t delay_spread(const int32_t* d, int64_t nb, int32_t ck, int G = dedisp_group_trials()) {
     int32_t sp = 0;
+    std::vector<int32_t> lo(ck), hi(ck);
     for (int64_t g = 0; g < nb; g += G) {
         const int64_t ge = std::min<int64_t>(nb, g + G);
-        for (int32_t c = 0; c < ck; ++c) {
-            int32_t lo = d[g * ck + c], hi = lo;
-            for (int64_t i = g + 1; i < ge; ++i) {
-                lo = std::min(lo, d[i * ck + c]);
-                hi = std::max(hi, d[i * ck + c]);
+        std::copy(d + g * ck, d + (g + 1) * ck, lo.begin());
+        std::copy(d + g * ck, d + (g + 1) * ck, hi.begin());
+        for (int64_t i = g + 1; i < ge; ++i) {
+            const int32_t* di = d + i * ck;
+            for (int32_t c = 0; c < ck; ++c) {
+                lo[c] = std::min(lo[c], di[c]);
+                hi[c] = std::max(hi[c], di[c]);
             }
-            sp = std::max(sp, hi - lo);
         }
+        for (int32_t c = 0; c < ck; ++c) sp = std::max(sp, hi[c] - lo[c]);
     }
     return sp;
 }
@@ -414,29 +437,27 @@ void dd_choose(const Tune& tune, const pss_fil_desc* fil, const StageInfo& st, c
     }
     if (bx_use(tune, st.ds) && ck <= 65535) return;
     if (st.ds > 64 || nb < 8) return;
-    DdTables t;
-    if (!dd_tables(delays, nb, ck, &t)) return;
     // Shared sums where they take at most 1.2 shared-memory wavefronts per channel, trial and 128 samples (the
     // direct kernel: 1, and five instructions).  Measured: 0.95 (256 channels, 0.5 pc cm^-3 steps) 2.45 against
     // 3.91 ms, 1.14 (1 pc cm^-3 steps) 1.23 against 1.57 ms, 1.31 (64 channels, where most of 32 trials have
     // patterns of their own) 54.7 against 51.2 us.
-    if (t.cost > 1.2 * (double)nb * ck) return;
+    DdTables t;
+    if (!dd_tables(delays, nb, ck, 1.2, host, &t)) return;
     d->kind = DD_SHARED;
-    d->off = (host->size() + 255) & ~size_t(255);
+    d->off = t.off;
     d->chunk_off = t.chunk_off;
     d->chan_off = t.chan_off;
-    host->resize(d->off + t.bytes.size());
-    memcpy(host->data() + d->off, t.bytes.data(), t.bytes.size());
 }
 
-// Put the batches' tables on the device (waits: `host` is the caller's).  The
-// set-up kept for that buffer goes first: its tables are overwritten.
-pss_status dd_upload(pss_ctx* ctx, int which, const std::vector<uint8_t>& host, cudaStream_t s) {
+// Put the batches' tables (ctx->dd_host) on the device.  The set-up kept for
+// that buffer goes first: its tables are overwritten.
+pss_status dd_upload(pss_ctx* ctx, int which, Uploads* up) {
+    const std::vector<uint8_t>& host = ctx->dd_host;
     if (host.empty()) return PSS_OK;
     (which == 0 ? ctx->path_cache : ctx->dd_cache).reset();
     PSS_TRY(ctx->ddtab[which].ensure(host.size()));
-    PSS_CUDA(cudaMemcpyAsync(ctx->ddtab[which].p, host.data(), host.size(), cudaMemcpyHostToDevice, s));
-    PSS_CUDA(cudaStreamSynchronize(s));
+    up->pending = true;
+    PSS_CUDA(cudaMemcpyAsync(ctx->ddtab[which].p, host.data(), host.size(), cudaMemcpyHostToDevice, up->s));
     return PSS_OK;
 }
 
@@ -926,10 +947,10 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
         return PSS_OK;
     }
     auto D = std::make_shared<DdSetup>();
-    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T));
+    Uploads up(s);
+    ctx->dd_host.clear();
+    PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &D->ck, &D->pitch, &D->T, &up));
     D->need_bytes = D->T.on;
-    const std::vector<int32_t> hd = D->T.on ? std::vector<int32_t>() : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
-    std::vector<uint8_t> dd_host;
     int64_t off = 0;
     for (size_t si = 0; si < plan->stages.size(); ++si) {
         const StageInfo& st = plan->stages[si];
@@ -951,9 +972,9 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
                 d.sub = sub_batch(plan, D->T, D->ck, dm_begin, b0, d.nb, st.nv, st.ds);
                 D->need_subu = std::max(D->need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
             } else {
-                const int32_t* rows = hd.data() + (size_t)(b0 - dm_begin) * D->ck;
-                d.spread = delay_spread(rows, d.nb, D->ck);
-                dd_choose(ctx->tune, fil, st, rows, d.nb, D->ck, 1, &dd_host, &d.dd);
+                const int32_t* rows = ctx->delays_host.data() + D->ck + (size_t)(b0 - dm_begin) * D->ck;
+                dd_choose(ctx->tune, fil, st, rows, d.nb, D->ck, 1, &ctx->dd_host, &d.dd);
+                if (d.dd.kind == DD_DIRECT) d.spread = delay_spread(rows, d.nb, D->ck);
                 (d.dd.kind == DD_BITS ? D->need_bits : D->need_bytes) = true;
             }
             d.out_off = off;
@@ -962,7 +983,8 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
         }
     }
     if (D->need_subu) PSS_TRY(ctx->subu.ensure(D->need_subu));
-    PSS_TRY(dd_upload(ctx, 1, dd_host, s));
+    PSS_TRY(dd_upload(ctx, 1, &up));
+    PSS_TRY(up.wait());
     D->key.swap(key);
     D->gen = ctx->delays_gen;
     ctx->dd_cache = D;
@@ -976,6 +998,7 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
     std::string key = path_key(plan, fil, cfg, dm_begin, dm_end, mode, dev_cap, max_b, ctx->tune);
     PathCache* pc = static_cast<PathCache*>(ctx->path_cache.get());
     const bool hit = pc && pc->key == key && dm_end > dm_begin;
+    Uploads up(s);
     if (hit) {
         if (pc->gen != ctx->delays_gen) {  // another request's delays are on the device; the rest still stands
             SubTab T;
@@ -986,7 +1009,8 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
         PSS_TRY(ensure_unpacked(ctx, fil, pc->P.ck, pc->P.pitch, pc->P.need_bytes, pc->P.need_bits));
         *P = pc->P;
     } else {
-        PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &P->ck, &P->pitch, &P->sub));
+        ctx->dd_host.clear();
+        PSS_TRY(setup_input(ctx, plan, fil, dm_begin, dm_end, s, &P->ck, &P->pitch, &P->sub, &up));
     }
     if (!hit) {
         P->batches.clear();
@@ -995,13 +1019,11 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
     P->dev_cap = dev_cap;
     // (MODE_GAINS: the refinement also reads the byte rows, channel by channel)
     if (!hit) P->need_bytes = P->sub.on || mode == MODE_GAINS || dm_end == dm_begin;
-    if (dm_end == dm_begin) return PSS_OK;
+    if (dm_end == dm_begin) return up.wait();
     PSS_TRY(ensure_templates(ctx, cfg, s));
     P->nz = nz_of(cfg);
     P->Z = cfg->zmax ? (int)llround(cfg->zmax / cfg->dz) : 0;
     P->nstages = (int)log2((double)cfg->numharm) + 1;
-    const std::vector<int32_t> hd = (hit || P->sub.on) ? std::vector<int32_t>()
-                                                       : compact_delays(plan, kept_channels(fil), dm_begin, dm_end);
     if (mode == MODE_SEARCH) {
         PSS_TRY(ctx->cands.ensure((size_t)dev_cap * sizeof(pss_raw_cand)));
         PSS_TRY(ctx->counter.ensure(sizeof(unsigned long long)));
@@ -1019,7 +1041,6 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
         if (st.n_dm > 0) PSS_TRY(ensure_passtw(ctx, st.nfft / 2, ctx->tune.split_for(st.nfft / 2), s));
     size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, need_subu = 0;
     int64_t out_off = 0;
-    std::vector<uint8_t> dd_host;
     if (hit) {
         need_series = pc->need[0];
         need_fft = pc->need[1];
@@ -1050,7 +1071,7 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
         need_fft = std::max(need_fft, (size_t)B * M * 8);
         if (mode == MODE_SEARCH) need_plane = std::max(need_plane, (size_t)B * P->nz * nfft * 4);
         for (int64_t b0 = lo; b0 < hi; b0 += B) {
-            BatchDesc d;
+            BatchDesc d{};
             d.stage = (int32_t)si;
             d.b0 = b0;
             d.nb = (int32_t)std::min<int64_t>(B, hi - b0);
@@ -1059,9 +1080,9 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
                 d.sub = sub_batch(plan, P->sub, P->ck, dm_begin, b0, d.nb, st.nv, st.ds);
                 need_subu = std::max(need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
             } else {
-                const int32_t* rows = hd.data() + (size_t)(b0 - dm_begin) * P->ck;
-                d.spread = delay_spread(rows, d.nb, P->ck);
-                dd_choose(ctx->tune, fil, st, rows, d.nb, P->ck, 0, &dd_host, &d.dd);
+                const int32_t* rows = ctx->delays_host.data() + P->ck + (size_t)(b0 - dm_begin) * P->ck;
+                dd_choose(ctx->tune, fil, st, rows, d.nb, P->ck, 0, &ctx->dd_host, &d.dd);
+                if (d.dd.kind == DD_DIRECT) d.spread = delay_spread(rows, d.nb, P->ck);
                 (d.dd.kind == DD_BITS ? P->need_bits : P->need_bytes) = true;
             }
             d.out_off = out_off;
@@ -1069,7 +1090,8 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
             P->batches.push_back(d);
         }
     }
-    if (!hit) PSS_TRY(dd_upload(ctx, 0, dd_host, s));
+    if (!hit) PSS_TRY(dd_upload(ctx, 0, &up));
+    PSS_TRY(up.wait());
     PSS_TRY(ctx->series.ensure(need_series));
     if (need_subu) PSS_TRY(ctx->subu.ensure(need_subu));
     PSS_TRY(ctx->sums.ensure(need_sums));

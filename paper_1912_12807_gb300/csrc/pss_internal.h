@@ -198,6 +198,7 @@ struct Ctx {
     std::vector<int32_t> fold_host;    // what fold_tab holds, empty if unknown
     DevBuf xbits;        // rows of bits of a 1-bit file (bit-sliced dedispersion)
     DevBuf ddtab[2];     // tables of the shared-sum dedispersion: the search path's batches, the plain calls'
+    std::vector<uint8_t> dd_host;  // the tables under construction (kept for its memory)
     DevBuf series;       // float [B][nfft]
     DevBuf sums;         // unsigned long long [B]
     DevBuf fftA, fftB;   // float2 [B][M]
@@ -386,20 +387,21 @@ static_assert(sizeof(DdChunk) == 64, "a multiple of 16 bytes");
 constexpr int DD_BLOBHEAD = 2 * sizeof(DdChunk) + DD_MAXUNITS * 4 * 8;
 struct DdTables {
     int ngroups = 0;
-    size_t chunk_off = 0, chan_off = 0;
-    double cost = 0;             // estimated shared-memory accesses (host_dedisp.cpp)
-    std::vector<uint8_t> bytes;  // what the kernel reads
+    size_t off = 0;                       // of the tables in `host`
+    size_t chunk_off = 0, chan_off = 0;   // from there
+    double cost = 0;                      // estimated shared-memory accesses (host_dedisp.cpp)
 };
-// Tables of nb trials with delays [nb][ck]; false where a delay spread does
-// not fit the kernel's shared memory.
-bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, DdTables* out);
+// Tables of nb trials with delays [nb][ck], appended to `host`; false where
+// they cost more than max_cost per trial and channel, or where a delay spread
+// does not fit the kernel's shared memory.
+bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, double max_cost, std::vector<uint8_t>* host, DdTables* out);
 // Device bytes the tables of n trials in batches of nb can take at most.
 size_t dd_tables_bound(int64_t n, int64_t ck, int64_t nb);
 struct DdArgs {
     const uint8_t* xcm;
     int64_t pitch;
     int32_t ck;
-    const uint8_t* tab;          // DdTables::bytes on the device (16-byte aligned)
+    const uint8_t* tab;          // the tables on the device (16-byte aligned)
     size_t chunk_off, chan_off;
     int32_t nb;
     int64_t nv;                  // outputs per trial
