@@ -246,8 +246,9 @@ struct Uploads {
 
 // Host-side set-up for a file: the kept channels, their delays for
 // [dm_begin, dm_end) (or the two-stage tables, `T`) uploaded to
-// ctx->delays_dev, and the channel-major buffer.  Synchronises `s` (the
-// delay upload reads a host vector), or leaves that to `up`.
+// ctx->delays_dev.  Synchronises `s` (the delay upload reads a host vector),
+// or leaves that to `up`.  The unpacked file's buffers are the caller's
+// (ensure_unpacked): which are needed depends on how its trials are dedispersed.
 pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil, int64_t dm_begin,
                        int64_t dm_end, cudaStream_t s, int32_t* ck_out, int64_t* pitch_out, SubTab* T = nullptr,
                        Uploads* up = nullptr) {
@@ -290,8 +291,6 @@ pss_status setup_input(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* f
                                  cudaMemcpyHostToDevice, s));
         ctx->delays_gen++;
     }
-    PSS_TRY(ctx->xcm.ensure((size_t)ck * pitch + 64));
-    if (fil->nbits == 1 && plan->nsub == 0 && ck <= 255) PSS_TRY(ctx->xbits.ensure(b1_bytes(ck, fil->nsamp)));
     PSS_TRY(ensure_bx(ctx, plan, ck, dm_begin, dm_end));
     PSS_TRY(ensure_errflag(ctx, s));
     PSS_TRY(own.wait());
@@ -982,6 +981,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
             D->batches.push_back(d);
         }
     }
+    PSS_TRY(ensure_unpacked(ctx, fil, D->ck, D->pitch, D->need_bytes, D->need_bits));
     if (D->need_subu) PSS_TRY(ctx->subu.ensure(D->need_subu));
     PSS_TRY(dd_upload(ctx, 1, &up));
     PSS_TRY(up.wait());
@@ -1019,7 +1019,10 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
     P->dev_cap = dev_cap;
     // (MODE_GAINS: the refinement also reads the byte rows, channel by channel)
     if (!hit) P->need_bytes = P->sub.on || mode == MODE_GAINS || dm_end == dm_begin;
-    if (dm_end == dm_begin) return up.wait();
+    if (dm_end == dm_begin) {
+        PSS_TRY(ensure_unpacked(ctx, fil, P->ck, P->pitch, P->need_bytes, P->need_bits));
+        return up.wait();
+    }
     PSS_TRY(ensure_templates(ctx, cfg, s));
     P->nz = nz_of(cfg);
     P->Z = cfg->zmax ? (int)llround(cfg->zmax / cfg->dz) : 0;
@@ -1090,7 +1093,10 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
             P->batches.push_back(d);
         }
     }
-    if (!hit) PSS_TRY(dd_upload(ctx, 0, &up));
+    if (!hit) {
+        PSS_TRY(ensure_unpacked(ctx, fil, P->ck, P->pitch, P->need_bytes, P->need_bits));
+        PSS_TRY(dd_upload(ctx, 0, &up));
+    }
     PSS_TRY(up.wait());
     PSS_TRY(ctx->series.ensure(need_series));
     if (need_subu) PSS_TRY(ctx->subu.ensure(need_subu));
@@ -2301,6 +2307,7 @@ pss_status pss_fold(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fil,
     const int32_t* tab = nullptr;  // exact plans: the kept channels and the delays of the runs' trials
     if (plan->nsub > 0) {
         PSS_TRY(setup_input(ctx, plan, fil, lo_dm, hi_dm + 1, s, &ck, &pitch, &T));
+        PSS_TRY(ensure_unpacked(ctx, fil, ck, pitch, true, false));
     } else {
         // a table of the folded trials alone, beside the one that searches and dedispersions keep
         const std::vector<int32_t> keep = kept_channels(fil);
@@ -3111,11 +3118,28 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
         const size_t ng = plan.grp_first.size();
         tables = std::max(tables, (size_t)ck + ng * ck + (size_t)plan.ndm() * plan.nsub + 2 * ng + 2 * plan.nsub + 16);
     }
-    size_t t = buf((size_t)file_bytes(fil)) + buf((size_t)ck * pitch + 64) +
-               (fil->nbits == 1 && plan.nsub == 0 && ck <= 255 ? buf(b1_bytes(ck, fil->nsamp)) : 0) + buf(tables * sizeof(int32_t)) +
+    // 1-bit files: rows of bits, and rows of bytes unless the bit-sliced kernel takes every trial for certain, however
+    // the trials fall into its groups (delays grow fastest in the channel whose delays are largest; 2 for rounding)
+    const bool bits = fil->nbits == 1 && plan.nsub == 0 && ck <= 255;
+    bool bytes = true;
+    if (bits && plan.ndm() > 0) {
+        const int32_t* last = &plan.delays[(size_t)(plan.ndm() - 1) * plan.nchan];
+        const int32_t c = *std::max_element(keep.begin(), keep.end(), [&](int32_t a, int32_t b) { return last[a] < last[b]; });
+        int32_t spread = 0;
+        for (const auto& st : plan.stages)
+            for (int64_t i = st.first; i < st.first + st.n_dm; ++i) {
+                const int64_t e = std::min<int64_t>(i + 31, st.first + st.n_dm - 1);
+                spread = std::max(spread, std::abs(plan.delays[(size_t)e * plan.nchan + c] - plan.delays[(size_t)i * plan.nchan + c]));
+            }
+        int KW, rowb;
+        size_t shm;
+        bytes = !b1_sizes(spread + 2, (int32_t)ck, 32, &KW, &rowb, &shm);
+    }
+    size_t t = buf((size_t)file_bytes(fil)) + (bytes ? buf((size_t)ck * pitch + 64) : 0) +
+               (bits ? buf(b1_bytes(ck, fil->nsamp)) : 0) + buf(tables * sizeof(int32_t)) +
                buf(sizeof(int)) + buf((size_t)dev_cap * sizeof(pss_raw_cand)) + buf(sizeof(unsigned long long));
     int64_t nfft_max = 0, total_taps = 0;
-    size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, subu = 0, bx = 0, ddt = 0;
+    size_t need_series = 0, need_fft = 0, need_sums = 0, need_plane = 0, subu = 0, bx = 0, ddt = 0, spare = 0;
     Tune bx_tune;  // the boxcar-table threshold a new context takes (environment included)
     if (const char* f = getenv("PSS_DEDISP_BX_MIN")) bx_tune.bx_min = std::max(0, atoi(f));
     std::vector<int64_t> sizes;
@@ -3128,8 +3152,15 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
             t += buf((size_t)(st.nfft / 2) * sizeof(float2));  // inter-pass twiddles (at most M entries)
         }
         const int64_t B = batch_trials(st.nfft, nz, MODE_SEARCH, st.n_dm);
-        // shared-sum tables of the stage's batches (at most; batches may be smaller than B)
-        if (plan.nsub == 0) ddt += dd_tables_bound(st.n_dm, ck, std::min<int64_t>(B, std::max<int64_t>(1, pipeline_batch(plan.ndm()))));
+        // shared-sum tables of the stage's batches (rows of 8 and more come from the boxcar table instead).  A batch runs
+        // fewer than B trials at once where the plan has more than 256 (DM batches of 30 %, launch shapes timed on 256):
+        // what is left of the buffers for B is more than the tables take
+        const int64_t most = std::max<int64_t>(256, pipeline_batch(plan.ndm()));
+        if (fil->nbits == 8 && plan.nsub == 0 && st.ds < Tune().bx_min) {
+            const int64_t per = std::min<int64_t>(B, std::max<int64_t>(1, pipeline_batch(plan.ndm()) > 0 ? pipeline_batch(plan.ndm()) : B));
+            for (int64_t b = 0; b < st.n_dm; b += per) ddt += dd_tables_bound(std::min<int64_t>(per, st.n_dm - b), ck) + 256;
+        }
+        if (B > most) spare = std::max(spare, (size_t)(B - most) * st.nfft * 4);
         if (plan.nsub > 0) {
             // stage-1 rows: groups touched by a batch x subbands x (N_v ds + largest D, padded)
             const int64_t ngb = (B + plan.sub_group - 1) / plan.sub_group + 1;
@@ -3149,7 +3180,7 @@ size_t search_footprint(const Plan& plan, const pss_fil_desc* fil, const pss_sea
         t += buf((size_t)nz * 2 * PLANE_FFT_L * sizeof(float2));
     t += buf((size_t)nfft_max * sizeof(float2)) + buf(need_series) + buf(need_sums) + 3 * buf(need_fft) +
          buf(need_plane) + buf((size_t)total_taps * sizeof(float2)) + buf((size_t)5 * nz * sizeof(int32_t)) +
-         buf(subu) + buf(bx) + buf(ddt);
+         buf(subu) + buf(bx) + (buf(ddt) > spare ? buf(ddt) - spare : 0);
     return t;
 }
 

@@ -334,6 +334,7 @@ bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, double max_cost, s
     out->chunk_off = (size_t)ng * sizeof(int4);
     out->chan_off = out->chunk_off + nchunk * sizeof(DdChunk);
     const size_t blob0 = (out->chan_off + (size_t)ng * ck * sizeof(int2) + 15) & ~size_t(15);
+    if (blob0 + nblob > dd_tables_bound(nb, ck)) return false;
     host->resize(out->off + blob0 + nblob);
     uint8_t* B = host->data() + out->off;
     size_t ci = 0, bo = blob0;
@@ -354,10 +355,7 @@ bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, double max_cost, s
     return true;
 }
 
-size_t dd_tables_bound(int64_t n, int64_t ck, int64_t nb) {
-    const int64_t batches = (n + nb - 1) / nb, groups = n / GT + batches;
-    // per channel at most one unit and one chunk: a row and a pair per trial, a chunk record, a channel entry
-    return (size_t)groups * (sizeof(int4) + (size_t)ck * (GT * 28 + 16 + sizeof(DdChunk) + sizeof(int2))) + (size_t)batches * 512;
-}
+// (tables that gain take 2.2 to 6.5 bytes per trial and channel)
+size_t dd_tables_bound(int64_t nb, int64_t ck) { return (size_t)(8 * nb * ck) + 16384; }
 
 }  // namespace pss

@@ -395,8 +395,9 @@ struct DdTables {
 // they cost more than max_cost per trial and channel, or where a delay spread
 // does not fit the kernel's shared memory.
 bool dd_tables(const int32_t* delays, int64_t nb, int32_t ck, double max_cost, std::vector<uint8_t>* host, DdTables* out);
-// Device bytes the tables of n trials in batches of nb can take at most.
-size_t dd_tables_bound(int64_t n, int64_t ck, int64_t nb);
+// Bytes that the tables of one batch of nb trials can take at most (dd_tables
+// refuses larger ones; a batch's tables start on a 256-byte boundary).
+size_t dd_tables_bound(int64_t nb, int64_t ck);
 struct DdArgs {
     const uint8_t* xcm;
     int64_t pitch;
