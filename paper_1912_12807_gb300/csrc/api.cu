@@ -3018,6 +3018,15 @@ pss_status autotune(pss_ctx* ctx, const Plan& plan, const pss_fil_desc* fil, con
         ctx->tune = Tune();
         return st;
     }
+    // the inter-pass tables of the splits that were tried and not taken (every pass over them has been waited for)
+    for (auto it = ctx->passtw.begin(); it != ctx->passtw.end();) {
+        if (it->variant == ctx->tune.split_for(it->M)) {
+            ++it;
+        } else {
+            it->buf.release();
+            it = ctx->passtw.erase(it);
+        }
+    }
     std::lock_guard<std::mutex> g(g_tune_mu);
     g_tuned.emplace(key, ctx->tune);
     return PSS_OK;
