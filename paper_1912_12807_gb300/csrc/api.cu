@@ -3011,8 +3011,26 @@ pss_status autotune(pss_ctx* ctx, const Plan& plan, const pss_fil_desc* fil, con
         }
         if (st == PSS_OK && cfg->zmax > 0 && plane_fft_usable(cfg->zmax, cfg->halfwidth_extra, plan.stages[0].nfft / 2))
             st = sweep(&ctx->tune.plane_form, {1, 0}, 1u << 4, "plane form");
-        if (st == PSS_OK) st = sweep(&ctx->tune.harm_run, {8, 16}, 1u << 5, "harm run");
-        if (st == PSS_OK) st = sweep(&ctx->tune.dedisp_kb, {96, 64}, 1u << 1, "dedisp kb");
+        if (st == PSS_OK) {
+            // choices that no kernel of the timed trials depends on are left at their defaults: the points per lane
+            // where every batch takes tiles of rows, the staging budget where none is dedispersed directly
+            PathSetup T;
+            st = setup_path(ctx, pp, fil, cfg, tb, te, MODE_SEARCH, s, kBatchInitialCap, &T);
+            bool run = false, kb = false;
+            for (const BatchDesc& d : T.batches) {
+                const StageInfo& sg = plan.stages[d.stage];
+                HarmArgs ha{};
+                ha.nfft = sg.nfft;
+                ha.nz = T.nz;
+                ha.Z = T.Z;
+                ha.nb = d.nb;
+                ha.nstages = T.nstages;
+                run |= !harm_takes_tiles(ha);
+                kb |= T.sub.on || (d.dd.kind == DD_DIRECT && !(bx_use(ctx->tune, sg.ds) && T.ck <= 65535 && d.nb >= 16));
+            }
+            if (st == PSS_OK && run) st = sweep(&ctx->tune.harm_run, {8, 16}, 1u << 5, "harm run");
+            if (st == PSS_OK && kb) st = sweep(&ctx->tune.dedisp_kb, {96, 64}, 1u << 1, "dedisp kb");
+        }
     }
     if (st != PSS_OK) {
         ctx->tune = Tune();

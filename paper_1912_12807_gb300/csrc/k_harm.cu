@@ -484,10 +484,14 @@ cudaError_t launch_reg(const HarmArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+bool harm_takes_tiles(const HarmArgs& a) {
+    return harm_rows() && tile_usable(a) && (harm_rows() == 1 || tile_gains(a));
+}
+
 cudaError_t launch_harm(const HarmArgs& a, cudaStream_t s) {
     if (a.nfft > (int64_t(1) << 24) || a.nstages > 6) return cudaErrorInvalidValue;
     if ((int64_t)a.nz * a.nfft > (int64_t(1) << 31)) return cudaErrorInvalidValue;  // 32-bit plane offsets
-    if (harm_rows() && tile_usable(a) && (harm_rows() == 1 || tile_gains(a))) return launch_tile(a, s);
+    if (harm_takes_tiles(a)) return launch_tile(a, s);
     // register-blocked kernel: up to 16 harmonics, whole warps of 32 x 16 points
     if (a.run == 8 && a.nstages <= 5 && a.nfft % (REG_NT * 8) == 0 && a.nfft / (REG_NT * 8) <= 65535 &&
         a.nb <= 65535)

@@ -712,6 +712,8 @@ struct HarmArgs {
     const int32_t* row_hmin;
 };
 cudaError_t launch_harm(const HarmArgs& a, cudaStream_t s);
+// whether it sums tiles of rows (shape fields alone), where `run` has no effect
+bool harm_takes_tiles(const HarmArgs& a);
 
 
 struct RefinePt {
