@@ -207,6 +207,9 @@ __global__ void __launch_bounds__(NT, 2) k_dedisp_b1(const __grid_constant__ B1A
     __syncthreads();
     if (threadIdx.x == 0) mbar_expect_tx(bar, (uint32_t)(a.ck * a.rowb));
     __syncthreads();
+    // (a limit of one poll, which tests set to see the wait run out, takes it here: after the offsets below the copies
+    // have mostly landed)
+    const bool in_time = a.wait_polls != 1 || warp != 0 || mbar_wait(bar, 0, 1);
     // channel c: the earliest delay of the group's trials, from a 16-byte boundary (128 samples), on
     bool bad = false;
     for (int c = threadIdx.x; c < a.ckp; c += NT) {
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(NT, 2) k_dedisp_b1(const __grid_constant__ B1A
     }
     for (int i = threadIdx.x; i < KW * 32 + 4; i += NT) reinterpret_cast<uint32_t*>(sm + zrow)[i] = 0u;
     const int any_bad = __syncthreads_or(bad);
-    const bool ok = warp == 0 ? mbar_wait(bar, 0, a.wait_polls) : true;
+    const bool ok = in_time && (warp != 0 || mbar_wait(bar, 0, a.wait_polls));
     if (__syncthreads_or(!ok) || any_bad) {
         // (any_bad: a spread larger than the launch was sized for)
         if (threadIdx.x == 0 && a.err) atomicExch(a.err, any_bad ? 2 : 1);
