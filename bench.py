@@ -275,11 +275,11 @@ def stage_work(plan, wl, fil_nbytes):
     """Algorithmic work of one step per profiled stage: (bound, amount, unit).
 
     dedisperse: kept channels x output samples x ds additions (each output
-    sample sums one 8-bit sample per channel per native sample), two 16-bit
-    SWAR additions per 32-bit add; rows that dedisperse from the boxcar table
-    add one 16-bit table term per channel and output sample with one 32-bit
-    add, counted as the two SWAR slots it takes; bxtable: the table builds;
-    unpack: file read + channel-major write; fft: every pass reads and writes
+    sample sums one 8-bit sample per channel per native sample); rows that
+    dedisperse from the boxcar table add one 16-bit table term per channel and
+    output sample, counted as two; bxtable: the table builds; unpack: file read
+    + channel-major write of bytes (kernel_work: what the search's kernels
+    write); fft: every pass reads and writes
     8 bytes per complex point; whiten: spectrum read + write (where the
     whitening and the zmax 0 plane run as one kernel, the stage reads the
     spectrum and writes the plane: the same bytes, and the plane stage has
@@ -354,11 +354,42 @@ def alu_denominators(probe):
     smem = probe["lds_bytes_per_s"]
     issue = probe["mix_per_s"] / DEDISP_INSTR_PER_ADD
     return {"channel_adds_per_s": min(smem, issue), "smem_bound_adds_per_s": smem,
-            "issue_bound_adds_per_s": issue, "int32_adds_per_s": probe["int32_adds_per_s"],
+            "issue_bound_adds_per_s": issue, "logic_per_s": probe["lop3_per_s"],
+            "int32_adds_per_s": probe["int32_adds_per_s"],
             "fp32_flops_per_s": probe["fp32_flops_per_s"]}
 
 
-def roofline_of(stage, bound, amount, unit, ms, launches, peaks, peak_kind, alu):
+def kernel_work(work, wl, fil_nbytes, forms):
+    """stage_work() for the kernels that the search launches (`forms`:
+    pss.pss_dedisp_forms): a 1-bit file whose trials are all counted
+    bit-sliced is unpacked to one bit per channel and sample."""
+    work = dict(work)
+    C, N = wl.fil.nchan, wl.fil.nsamp
+    by_bytes = forms["direct"] + forms["shared"] + forms["boxcar"] > 0
+    out = (float(C) * N if by_bytes else 0.0) + (float(C) * N / 8.0 if forms["bits"] > 0 else 0.0)
+    work["unpack"] = ("hbm", float(fil_nbytes) + out, "bytes")
+    return work
+
+
+# Bit-sliced counting of 1-bit samples, per channel-addition (k_dedisp_b1): two 32-bit shared-memory words and
+# one shift and 2.4 logic operations per 32 samples of a channel.
+BITS_SMEM_BYTES_PER_ADD = 8.0 / 32.0
+BITS_LOGIC_PER_ADD = 3.4 / 32.0
+
+
+def dedisp_floor_s(forms, alu):
+    """Seconds the dedispersion of one step cannot go below at the measured
+    rates, kernel by kernel: direct sums at alu_denominators' ceiling; boxcar
+    terms at the same with two slots each (2 bytes of table through L1 at the
+    shared-memory rate); shared sums by the shared-memory bytes that their
+    tables have them move; bit-sliced counting by the slower of its
+    shared-memory words and its logic operations."""
+    lds = alu["smem_bound_adds_per_s"]
+    return ((forms["direct"] + 2.0 * forms["boxcar"]) / alu["channel_adds_per_s"] + forms["shared_bytes"] / lds
+            + forms["bits"] * max(BITS_SMEM_BYTES_PER_ADD / lds, BITS_LOGIC_PER_ADD / alu["logic_per_s"]))
+
+
+def roofline_of(stage, bound, amount, unit, ms, launches, peaks, peak_kind, alu, forms=None):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     per_launch = amount / max(launches, 1)
     t = (ms / max(launches, 1)) / 1e3
@@ -367,6 +398,16 @@ def roofline_of(stage, bound, amount, unit, ms, launches, peaks, peak_kind, alu)
         peak = hbm * 1e9
         return {"kernel": stage, "bound": "hbm", "achieved": ach / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": ach / peak, "traffic": None, "peak_source": "hbm_gbs (%s)" % peak_kind}
+    if unit == "channel-adds" and forms and forms["shared"] + forms["bits"] > 0:
+        # a step's additions over the time that its kernels' own limits leave for them
+        adds = forms["direct"] + 2.0 * forms["boxcar"] + forms["shared"] + forms["bits"]
+        peak = adds / dedisp_floor_s(forms, alu)
+        names = [k for f, k in (("shared", "k_dedisp_sh"), ("bits", "k_dedisp_b1"), ("boxcar", "k_dedisp_bx"),
+                                ("direct", "k_dedisp")) if forms[f] > 0]
+        return {"kernel": stage, "bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12,
+                "unit": "T channel-adds/s", "frac": ach / peak, "traffic": None, "kernels": names,
+                "peak_source": "measured (pss_measure_peaks): shared-memory bytes of the shared-sum tables, words and "
+                               "logic operations of the bit-sliced counting, the direct kernel's ceiling elsewhere"}
     if unit == "channel-adds":
         peak = alu["channel_adds_per_s"]
         return {"kernel": stage, "bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12,
@@ -454,13 +495,14 @@ def measure_search(pss, wl, name, steps, warmup, local_rank, flush, stream, peak
         e2e_ms.append(1e3 * (t1 - t0))
     e2e = max_over_ranks(statistics.mean(e2e_ms), world, dev)
 
-    work = stage_work(plan, wl, fil.nbytes())
+    forms = pss.pss_dedisp_forms(plan, cfg, 0, ndm)
+    work = kernel_work(stage_work(plan, wl, fil.nbytes()), wl, fil.nbytes(), forms)
     rooflines = {}
     for st, (ms_st, n_st) in prof.items():
         if n_st == 0:
             continue
         bound, amount, unit = work[st]
-        rooflines[st] = roofline_of(st, bound, amount * psteps, unit, ms_st, n_st, peaks, peak_kind, alu)
+        rooflines[st] = roofline_of(st, bound, amount * psteps, unit, ms_st, n_st, peaks, peak_kind, alu, forms)
         if traffic:
             rooflines[st]["traffic"] = recorded_traffic(name, st)
     if "whiten" in rooflines and cfg.zmax == 0 and prof.get("plane", (0.0, 0))[1] == 0:
@@ -477,7 +519,7 @@ def measure_search(pss, wl, name, steps, warmup, local_rank, flush, stream, peak
         if bx_rows:
             rooflines["dedisperse"]["note"] = (
                 "rows with ds %s dedisperse from a per-channel boxcar table built once per ds (stage bxtable): "
-                "one table term per output and channel, a 32-bit add counted as two 16-bit SWAR slots" % bx_rows)
+                "one 2-byte table term per output and channel, counted as two slots of the ceiling" % bx_rows)
     dominant = max(prof, key=lambda k: prof[k][0])
     launches_per_step = sum(n for _, n in prof.values()) / psteps
     bi = fil.nbytes()
@@ -491,7 +533,7 @@ def measure_search(pss, wl, name, steps, warmup, local_rank, flush, stream, peak
            "gpu_launches": int(round(launches_per_step * steps)),
            "stages_ms_per_step": {k: v[0] / psteps for k, v in prof.items()},
            "stage_launches_per_step": {k: v[1] / psteps for k, v in prof.items()},
-           "stage_rooflines": {k: {kk: v[kk] for kk in ("bound", "frac", "achieved", "unit", "hbm_frac", "note")
+           "stage_rooflines": {k: {kk: v[kk] for kk in ("bound", "frac", "achieved", "unit", "hbm_frac", "note", "kernels")
                                    if kk in v} for k, v in rooflines.items()},
            "clocks": clocks.summary(), "wall_s_timed": t_wall, "candidates": int(len(cands))}
     return res, ctx, plan, cfg, data_dev, cands

@@ -616,6 +616,14 @@ pss_status pss_ctx_set_fft_split(pss_ctx* ctx, int64_t nfft, int32_t split);
  * arguments pss_batch_create would reject. */
 pss_status pss_search_footprint(const pss_plan* plan, const pss_fil_desc* fil, const pss_search_cfg* cfg,
                                 size_t* bytes);
+/* How a search of trials [dm_begin, dm_end) is dedispersed: kept channels x
+ * native samples added by each kernel in adds[4] (host): 0 directly, 1 with
+ * partial sums shared between trials, 2 bit-sliced 1-bit samples, 3 from the
+ * boxcar table (one term per channel and output sample); and the bytes of
+ * shared memory that kernel 1's tables have it move (*shared_bytes).
+ * Two-stage plans count as 0.  Computed on the host without a device. */
+pss_status pss_dedisp_forms(const pss_plan* plan, const pss_fil_desc* fil, const pss_search_cfg* cfg,
+                            int64_t dm_begin, int64_t dm_end, double* adds, double* shared_bytes);
 void pss_batch_free(pss_batch* b);
 
 /* ---- serving: continuous batching of files as they arrive --------------- */

@@ -416,6 +416,7 @@ struct DdBatch {
     int kind = DD_DIRECT;
     int which = 0;
     size_t off = 0, chunk_off = 0, chan_off = 0;
+    double cost = 0;                // shared sums: wavefronts per 128 samples of a tile
     int32_t spread = 0, group = 0;  // bit-sliced: trials per CTA and their delay spread
 };
 
@@ -446,6 +447,7 @@ void dd_choose(const Tune& tune, const pss_fil_desc* fil, const StageInfo& st, c
     d->off = t.off;
     d->chunk_off = t.chunk_off;
     d->chan_off = t.chan_off;
+    d->cost = t.cost;
 }
 
 // Put the batches' tables (ctx->dd_host) on the device.  The set-up kept for
@@ -3218,6 +3220,50 @@ extern "C" pss_status pss_search_footprint(const pss_plan* plan, const pss_fil_d
     if (!bytes) return fail(PSS_EINVAL, "pss_search_footprint: null argument");
     PSS_TRY(validate_search(plan, fil, cfg));
     *bytes = search_footprint(*plan, fil, cfg, kBatchInitialCap);
+    return PSS_OK;
+}
+
+extern "C" pss_status pss_dedisp_forms(const pss_plan* plan, const pss_fil_desc* fil, const pss_search_cfg* cfg,
+                                       int64_t dm_begin, int64_t dm_end, double* adds, double* shared_bytes) {
+    if (!adds || !shared_bytes) return fail(PSS_EINVAL, "pss_dedisp_forms: null argument");
+    PSS_TRY(check_common(reinterpret_cast<pss_ctx*>(1), plan, fil, fil, dm_begin, dm_end));
+    PSS_TRY(check_cfg(cfg, *plan));
+    for (int i = 0; i < 4; ++i) adds[i] = 0.0;
+    *shared_bytes = 0.0;
+    const std::vector<int32_t> keep = kept_channels(fil);
+    const int32_t ck = (int32_t)keep.size();
+    if (ck == 0) return fail(PSS_EINVAL, "channel mask removes every channel");
+    Tune tune;
+    if (const char* f = getenv("PSS_DEDISP_BX_MIN")) tune.bx_min = std::max(0, atoi(f));
+    const int64_t max_b = pipeline_batch(dm_end - dm_begin);
+    std::vector<uint8_t> host;
+    for (const StageInfo& st : plan->stages) {
+        const int64_t lo = std::max<int64_t>(dm_begin, st.first), hi = std::min<int64_t>(dm_end, st.first + st.n_dm);
+        if (lo >= hi) continue;
+        int64_t B = batch_trials(st.nfft, nz_of(cfg), MODE_SEARCH, hi - lo);
+        if (max_b > 0) B = std::min(B, max_b);
+        for (int64_t b0 = lo; b0 < hi; b0 += B) {
+            const int32_t nb = (int32_t)std::min<int64_t>(B, hi - b0);
+            const double per = (double)ck * nb * st.nv;
+            if (plan->nsub > 0) {
+                adds[0] += per * st.ds;
+                continue;
+            }
+            DdBatch d;
+            host.clear();
+            dd_choose(tune, fil, st, compact_delays(plan, keep, b0, b0 + nb).data(), nb, ck, 0, &host, &d);
+            if (d.kind == DD_BITS) {
+                adds[2] += per * st.ds;
+            } else if (d.kind == DD_SHARED) {
+                adds[1] += per * st.ds;
+                *shared_bytes += d.cost * (double)((st.nv * st.ds + DD_TN - 1) / DD_TN * DD_TN);
+            } else if (bx_use(tune, st.ds) && ck <= 65535 && (nb >= 16 || b0 > lo)) {
+                adds[3] += per;
+            } else {
+                adds[0] += per * st.ds;
+            }
+        }
+    }
     return PSS_OK;
 }
 

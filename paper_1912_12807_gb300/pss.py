@@ -68,7 +68,7 @@ EXPORTS = ["pss_ctx_create", "pss_ctx_destroy", "pss_last_error", "pss_version",
            "pss_search_raw", "pss_sift", "pss_sift_in_batches", "pss_search_dm_batch", "pss_response", "pss_sigma_of_power",
            "pss_power_threshold", "pss_ctx_profile", "pss_ctx_profile_read", "pss_dedisperse_noalloc",
            "pss_refine_prepare", "pss_refine_eval", "pss_refine_candidates", "pss_batch_create", "pss_batch_run",
-           "pss_batch_footprint", "pss_batch_free", "pss_search_footprint", "pss_ctx_take_cands",
+           "pss_batch_footprint", "pss_batch_free", "pss_search_footprint", "pss_dedisp_forms", "pss_ctx_take_cands",
            "pss_batch_take_cands", "pss_batch_tuning", "pss_batch_fft_split", "pss_fft_split_radices",
            "pss_ctx_set_fft_split", "pss_measure_peaks", "pss_ctx_set_wait_limit", "pss_debug_fail_alloc",
            "pss_ctx_check", "pss_search_multi", "pss_search_multi_footprint",
@@ -139,6 +139,7 @@ def lib():
         "pss_search_multi": (st, [vp, P(pss_search_cfg), vp, i32, C.c_int, vp, i64, vp, P(i64), vp]),
         "pss_search_multi_footprint": (st, [P(pss_search_cfg), vp, i32, P(C.c_size_t)]),
         "pss_search_footprint": (st, [vp, P(pss_fil_desc), P(pss_search_cfg), P(C.c_size_t)]),
+        "pss_dedisp_forms": (st, [vp, P(pss_fil_desc), P(pss_search_cfg), i64, i64, P(C.c_double), P(C.c_double)]),
         "pss_server_create": (st, [C.c_int, C.c_size_t, C.c_int, P(vp)]),
         "pss_server_create_grouped": (st, [C.c_int, C.c_size_t, C.c_int, C.c_int, P(vp)]),
         "pss_server_group_stats": (st, [vp, P(i64), P(i64)]),
@@ -681,6 +682,14 @@ def pss_ctx_set_fft_split(ctx: Context, nfft: int, split: int):
 
 def pss_batch_create(plan: Plan, cfg: pss_search_cfg, device: int = 0) -> Batch:
     return Batch(plan, cfg, device)
+
+
+def pss_dedisp_forms(plan: Plan, cfg: pss_search_cfg, dm_begin: int, dm_end: int) -> dict:
+    """How a search of [dm_begin, dm_end) is dedispersed: channel additions by kernel ("direct", "shared",
+    "bits", and "boxcar" table terms) and "shared_bytes", the shared-memory bytes of the "shared" kernel's tables."""
+    adds, b = (C.c_double * 4)(), C.c_double()
+    _check(lib().pss_dedisp_forms(plan.h, C.byref(plan.desc.c), C.byref(cfg), dm_begin, dm_end, adds, C.byref(b)))
+    return dict(zip(("direct", "shared", "bits", "boxcar"), (float(a) for a in adds)), shared_bytes=float(b.value))
 
 
 def pss_search_footprint(plan: Plan, cfg: pss_search_cfg) -> int:
