@@ -421,14 +421,14 @@ struct DdBatch {
 };
 
 // Choose a batch's kernel (delays [nb][ck]); shared-sum tables are appended to `host`.
-void dd_choose(const Tune& tune, const pss_fil_desc* fil, const StageInfo& st, const int32_t* delays, int32_t nb,
-               int32_t ck, int which, std::vector<uint8_t>* host, DdBatch* d) {
+void dd_choose(const Tune& tune, int num_sms, const pss_fil_desc* fil, const StageInfo& st, const int32_t* delays,
+               int32_t nb, int32_t ck, int which, std::vector<uint8_t>* host, DdBatch* d) {
     d->kind = DD_DIRECT;
     d->which = which;
     if (fil->nbits == 1) {
-        // 32 trials share a staged tile, 16 where that leaves fewer than two CTAs for each of about 150 SMs
+        // 32 trials share a staged tile, 16 where that leaves fewer than two CTAs per SM
         const int64_t tiles = (st.nv * st.ds + 4095) / 4096;
-        d->group = tiles * ((nb + 31) / 32) >= 300 ? 32 : 16;
+        d->group = tiles * ((nb + 31) / 32) >= 2 * (num_sms > 0 ? num_sms : 152) ? 32 : 16;
         d->spread = delay_spread(delays, nb, ck, d->group);
         int KW, rowb;
         size_t shm;
@@ -974,7 +974,7 @@ pss_status setup_dedisp(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* 
                 D->need_subu = std::max(D->need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
             } else {
                 const int32_t* rows = ctx->delays_host.data() + D->ck + (size_t)(b0 - dm_begin) * D->ck;
-                dd_choose(ctx->tune, fil, st, rows, d.nb, D->ck, 1, &ctx->dd_host, &d.dd);
+                dd_choose(ctx->tune, ctx->num_sms, fil, st, rows, d.nb, D->ck, 1, &ctx->dd_host, &d.dd);
                 if (d.dd.kind == DD_DIRECT) d.spread = delay_spread(rows, d.nb, D->ck);
                 (d.dd.kind == DD_BITS ? D->need_bits : D->need_bytes) = true;
             }
@@ -1086,7 +1086,7 @@ pss_status setup_path(pss_ctx* ctx, const pss_plan* plan, const pss_fil_desc* fi
                 need_subu = std::max(need_subu, (size_t)plan->nsub * d.sub.ngb * d.sub.stride1 * 4 + subsum_slack_bytes(d.sub.spread2));
             } else {
                 const int32_t* rows = ctx->delays_host.data() + P->ck + (size_t)(b0 - dm_begin) * P->ck;
-                dd_choose(ctx->tune, fil, st, rows, d.nb, P->ck, 0, &ctx->dd_host, &d.dd);
+                dd_choose(ctx->tune, ctx->num_sms, fil, st, rows, d.nb, P->ck, 0, &ctx->dd_host, &d.dd);
                 if (d.dd.kind == DD_DIRECT) d.spread = delay_spread(rows, d.nb, P->ck);
                 (d.dd.kind == DD_BITS ? P->need_bits : P->need_bytes) = true;
             }
@@ -3251,7 +3251,7 @@ extern "C" pss_status pss_dedisp_forms(const pss_plan* plan, const pss_fil_desc*
             }
             DdBatch d;
             host.clear();
-            dd_choose(tune, fil, st, compact_delays(plan, keep, b0, b0 + nb).data(), nb, ck, 0, &host, &d);
+            dd_choose(tune, 0, fil, st, compact_delays(plan, keep, b0, b0 + nb).data(), nb, ck, 0, &host, &d);
             if (d.kind == DD_BITS) {
                 adds[2] += per * st.ds;
             } else if (d.kind == DD_SHARED) {

@@ -21,13 +21,13 @@
 // k_dedisp_bx: a CTA owns GW consecutive trials (one warp each) and a tile
 // of TJ output samples; the lanes of a warp turn 32 channels' delays into
 // table offsets at once (ds is a power of two: a shift and a mask each) and
-// pass them round by shuffle.  A lane reads 32-bit words, two outputs of a
+// list them in shared memory, even element offsets first.  A lane reads 32-bit words, two outputs of a
 // channel each; words at an even and at an odd element offset are summed
 // apart (16-bit halves, widened before they can overflow) and combined, one
 // output shifted, at the end.  Adjacent trials mostly share a channel's phase
 // row and offset, so their warps read the same lines through L1.  Bound: the
-// latency of table reads that miss L1, so a warp sorts 32 channels by parity
-// and has the loads of four in flight at once.  979 trials of the six-row plan:
+// latency of table reads that miss L1 (long scoreboard; L1 at 31 %, DRAM at 23 %
+// of their rates), so a warp has the loads of four channels in flight at once.  979 trials of the six-row plan:
 // 1.35 ms with 16-bit loads, 1.22 ms with a branch per channel, 0.60 ms here.
 #include "pss_internal.h"
 

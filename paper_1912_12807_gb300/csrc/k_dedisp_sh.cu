@@ -21,8 +21,8 @@
 // 32-bit integers every 257 channels and added to by the same thread the
 // next time.
 //
-// Bound: shared-memory wavefronts (75 % of the cycles on the drift-scan plan,
-// 256 channels, 0.5 pc cm^-3 steps).  The direct kernel reads one byte per
+// Bound: shared-memory wavefronts (79 % of their rate on the drift-scan file, 256
+// channels, 0.5 pc cm^-3 steps; integer pipe 61 %).  The direct kernel reads one byte per
 // channel and trial and spends five instructions on four of them; here a
 // trial reads half a byte per channel, and a row costs 35 wavefronts per 640
 // sums.  32 trials x 512 samples leave two CTAs per SM (row forming of one

@@ -437,8 +437,9 @@ __global__ void __launch_bounds__(FNT, 3) k_plane_fft(const __grid_constant__ Pl
 // straight to the plane.
 //
 // Bound by the chain load - butterfly - barrier of a row with 16 warps per SM
-// (128 registers a thread), not by a unit: leaving out the template loads, the
-// twiddles, the arithmetic or the stores saves 5 to 16 % each.  The loop keeps
+// (128 registers a thread) and by shared memory (74 % of its rate in 8 trials x
+// 201 rows of 2^18; FMA pipe 26 %, DRAM 22 %): leaving out the template loads,
+// the twiddles, the arithmetic or the stores saves 5 to 16 % each.  The loop keeps
 // two pointers and its bins; even so 21 words are spilled in the set-up and 12
 // read back (ptxas: 84 bytes of spill stores, 48 of loads).  Template quads of
 // the next row loaded ahead, or the z = 0 row tested where its powers are
