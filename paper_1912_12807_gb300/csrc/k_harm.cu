@@ -244,25 +244,7 @@ __device__ __forceinline__ float harm_sum_ahead(const float* P, int h, int j, in
     return acc;
 }
 
-// The neighbours of (h, j) in the rows j - 1 and j + 1: whether s is above the one and not below the other.  The same
-// half-bin first (with interference, ridges over many rows: it decides most points), both rows' loads in flight.
-// Uncleaned files, rows / tiles with a chain of loads per neighbour / here: 32 trials x 101 rows of 2^18, 342 k
-// detections, 2.80 / 3.35 / 2.71 ms; 128 trials x 201 rows 28.9 / 32.5 / 25.6 ms.
-template <int SI>
-__device__ __forceinline__ bool beats_rows(const float* P, float s, int h, int j, int nfft, int nz, int Z) {
-    bool hit = true;
-#pragma unroll 1
-    for (int q = 0; q < 3 && hit; ++q) {
-        const int dh = q == 0 ? 0 : 2 * q - 3;
-        const float below = harm_sum_ahead<SI>(P, h + dh, j - 1, nfft, nz, Z);
-        const float above = harm_sum_ahead<SI>(P, h + dh, j + 1, nfft, nz, Z);
-        hit = s > below && s >= above;
-    }
-    return hit;
-}
-
-// TILE: called for the few warps of a tile with points above the threshold.
-template <int SI, int R, bool TILE = false>
+template <int SI, int R>
 __device__ __forceinline__ void reg_test(const HarmArgs& a, const float* P, const float (&acc)[R], int hw, int j,
                                          int lane, int b) {
     const float thr = a.thr[SI];
@@ -284,9 +266,7 @@ __device__ __forceinline__ void reg_test(const HarmArgs& a, const float* P, cons
             if (lane == 31) right = i < R - 1 ? r0 : harm_sum_at<SI>(P, hw + 32 * R, j, nfft, nz, Z);
             // strictly above every earlier neighbour, ties to the lower index against later ones
             bool hit = s > left && s >= right;
-            if (TILE) {
-                hit = hit && beats_rows<SI>(P, s, h, j, nfft, nz, Z);
-            } else if (nz > 1) {
+            if (nz > 1) {
 #pragma unroll
                 for (int dh = -1; dh <= 1; ++dh) {
                     if (!hit) break;
@@ -369,15 +349,71 @@ __global__ void __launch_bounds__(REG_NT) k_harm_reg(const __grid_constant__ Har
 // 2^18, 8 harmonics: 27.6 ms with one row per warp, 22.0 ms here; 1, 2 and 4
 // half-bins per thread 31.2, 23.1 and 22.0 ms (longer contiguous reads and more
 // of them in flight), 256 threads per block 22.3 ms.
-// The rare path: a warp with points of row j at or above the threshold.
+// The rare path: a warp with points of row j at or above the threshold (v: the lane's sums; vi, vo: those of the rows
+// one nearer to the centre row and one further, where the tile has them: bits 0 and 1 of `has`).  With interference it
+// is not rare and most points it sees are on a ridge over many rows, so what the tile's own sums rule out comes first,
+// and the loads of the sums it does not have are in flight together.  Uncleaned files, rows / tiles with a chain of
+// loads per neighbour / here: 32 trials x 101 rows of 2^18, 342 k detections, 2.80 / 3.35 / 2.56 ms; 128 trials x 201
+// rows 28.9 / 32.5 / 23.8 ms; a cleaned one 23.4 / 18.9 / 19.3 ms (held to 80 registers: 24.1 and 20.5 ms).
 template <int SI, int HP>
-__device__ __noinline__ void tile_hit(const HarmArgs& a, const float* P, float4 v, int hw, int j, int lane, int b) {
-    static_assert(HP <= 4, "points by value");
-    const float w[4] = {v.x, v.y, v.z, v.w};
-    float acc[HP];
+__device__ __noinline__ void tile_hit(const HarmArgs& a, float4 v, float4 vi, float4 vo, int has, int sgn, int d, int hw,
+                                      int b) {
+    static_assert(HP == 4, "points by value");
+    const float* P = a.plane + (int64_t)b * a.plane_stride;
+    const int lane = threadIdx.x & 31, j = a.Z + sgn * d;
+    const float4 vb = sgn > 0 ? vi : vo, va = sgn > 0 ? vo : vi;  // rows j - 1 and j + 1
+    const bool kb = has & (sgn > 0 ? 1 : 2), ka = has & (sgn > 0 ? 2 : 1);
+    const float thr = a.thr[SI], x[HP] = {v.x, v.y, v.z, v.w}, xb[HP] = {vb.x, vb.y, vb.z, vb.w}, xa[HP] = {va.x, va.y, va.z, va.w};
+    const int nfft = (int)a.nfft, hmin = a.row_hmin ? a.row_hmin[8 * b + SI] : a.hmin[SI], nz = a.nz, Z = a.Z;
 #pragma unroll
-    for (int i = 0; i < HP; ++i) acc[i] = w[i];
-    reg_test<SI, HP, true>(a, P, acc, hw, j, lane, b);
+    for (int i = 0; i < HP; ++i) {
+        // the points beside the lane's, in a row of sums; the warp's own first and last have none
+        auto beside = [&](const float (&r)[HP], float& l, float& u) {
+            l = __shfl_up_sync(0xffffffffu, r[i], 1);
+            u = __shfl_down_sync(0xffffffffu, r[i], 1);
+            const float l31 = __shfl_sync(0xffffffffu, r[i > 0 ? i - 1 : 0], 31);
+            const float u0 = __shfl_sync(0xffffffffu, r[i < HP - 1 ? i + 1 : HP - 1], 0);
+            if (lane == 0) l = l31;
+            if (lane == 31) u = u0;
+        };
+        float left, right, bl, br, al, ar;
+        beside(x, left, right);
+        beside(xb, bl, br);
+        beside(xa, al, ar);
+        const bool first = i == 0 && lane == 0, end = i == HP - 1 && lane == 31;
+        const float s = x[i];
+        const int h = hw + lane + 32 * i;
+        if (!(s >= thr && h >= hmin)) continue;
+        if (first) left = harm_sum_ahead<SI>(P, h - 1, j, nfft, nz, Z);
+        if (end) right = harm_sum_ahead<SI>(P, h + 1, j, nfft, nz, Z);
+        // strictly above every earlier neighbour, ties to the lower index against later ones
+        bool hit = s > left && s >= right;
+        if (kb) hit = hit && s > xb[i] && (first || s > bl) && (end || s > br);
+        if (ka) hit = hit && s >= xa[i] && (first || s >= al) && (end || s >= ar);
+        if (!(kb && ka && !first && !end)) {
+#pragma unroll 1
+            for (int q = 0; q < 3 && hit; ++q) {
+                const int dh = q == 0 ? 0 : 2 * q - 3;
+                const bool out = (first && dh < 0) || (end && dh > 0);
+                const float below = !kb || out ? harm_sum_ahead<SI>(P, h + dh, j - 1, nfft, nz, Z) : -INFINITY;
+                const float above = !ka || out ? harm_sum_ahead<SI>(P, h + dh, j + 1, nfft, nz, Z) : -INFINITY;
+                hit = s > below && s >= above;
+            }
+        }
+        if (hit) {
+            const unsigned long long slot = atomicAdd(a.counter, 1ull);
+            if ((int64_t)slot < a.cap) {
+                pss_raw_cand c;
+                c.dm_idx = a.row_dm ? a.row_dm[b] : a.dm0 + b;
+                c.numharm = 1 << SI;
+                c.h = h;
+                c.j = j;
+                c.power = s;
+                c.reserved = a.row_file ? a.row_file[b] : 0;
+                a.out[slot] = c;
+            }
+        }
+    }
 }
 
 template <int SI, int NSTAGES, int RT, int HP>
@@ -418,10 +454,11 @@ __device__ __forceinline__ void tile_stages(const HarmArgs& a, const char* Pz, i
 #pragma unroll
                 for (int i = 1; i < HP; ++i) m = fmaxf(m, acc[r][i]);
                 // (the centre row belongs to the side d >= 0)
-                if (r < nrow && (r > 0 || d0 > 0 || sgn > 0) && __any_sync(0xffffffffu, m >= a.thr[SI]))
-                    tile_hit<SI, HP>(a, a.plane + (int64_t)b * a.plane_stride, 
-                                     make_float4(acc[r][0], acc[r][HP > 1 ? 1 : 0], acc[r][HP > 2 ? 2 : 0], acc[r][HP > 3 ? 3 : 0]), hw,
-                                     a.Z + sgn * (d0 + r), lane, b);
+                if (r < nrow && (r > 0 || d0 > 0 || sgn > 0) && __any_sync(0xffffffffu, m >= a.thr[SI])) {
+                    auto row = [&](int q) { return make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]); };
+                    const int has = (r > 0 ? 1 : 0) | (r + 1 < RT && r + 1 < nrow ? 2 : 0);
+                    tile_hit<SI, HP>(a, row(r), row(r > 0 ? r - 1 : 0), row(r + 1 < RT ? r + 1 : r), has, sgn, d0 + r, hw, b);
+                }
             }
         }
         tile_stages<SI + 1, NSTAGES, RT, HP>(a, Pz, rstep, ta, acc, hw, nrow, sgn, d0, lane, b);
