@@ -301,8 +301,10 @@ void sort_raw(std::vector<pss_raw_cand>* v, int64_t ndm) {
     std::vector<std::pair<int64_t, int64_t>> bk;
     bucket_by_dm(v->data(), (int64_t)v->size(), ndm, &order, &bk);
     std::vector<pss_raw_cand> out(v->size());
-    for (size_t i = 0; i < order.size(); ++i) out[i] = (*v)[(size_t)order[i]];
-    parallel_for((int64_t)bk.size(), 8, [&](int64_t b) {
+    // long lists a trial per task, gathered and sorted (1.06 M detections of 64 trials in the order of the row tiles:
+    // with eight trials per task and the gather before them 69 ms for the call, 42 ms here)
+    parallel_for((int64_t)bk.size(), v->size() >= (size_t)1 << 16 ? 1 : 8, [&](int64_t b) {
+        for (int64_t i = bk[(size_t)b].first; i < bk[(size_t)b].second; ++i) out[(size_t)i] = (*v)[(size_t)order[(size_t)i]];
         std::sort(out.begin() + bk[(size_t)b].first, out.begin() + bk[(size_t)b].second,
                   [](const pss_raw_cand& x, const pss_raw_cand& y) {
                       if (x.numharm != y.numharm) return x.numharm < y.numharm;
